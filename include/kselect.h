@@ -193,7 +193,11 @@ int32_t select_kernel(gemm_handle_t handle, int64_t M, int64_t N, int64_t K, int
 
 /* ---------------------------------------------------------------- GEMM
  * C = alpha * op(A) * op(B) + beta * C for each batch entry, with the kernel
- * select_kernel() picks.  A and B are float* for F32/TF32/F32X3 handles and
+ * select_kernel() picks; where an FP32 SIMT or split-K choice is expected to
+ * be slower than the tensor cores running the same product at FP32 accuracy
+ * (every operand split exactly into three BF16 parts, six products, K chunks
+ * summed in FP32; see kselect_f32tc_selftest), gemm() and the other calls
+ * with a handle run that.  gemm_with_config and its kin run the config named. A and B are float* for F32/TF32/F32X3 handles and
  * bf16 (uint16_t*) for BF16 handles.  M, N or batch == 0 is a no-op; K == 0
  * sets C = beta * C.  When beta == 0, C is only written (it may hold NaN).
  * Sizes must be < 2^31 and batch <= 65535 (else GEMM_ERR_UNSUPPORTED). */
@@ -664,6 +668,22 @@ gemm_status_t gemm_device_status(int32_t* out_status, int32_t clear);
  * *waited_out = 0 (1 would mean the barrier completed).  The context stays
  * usable.  Synchronises `stream`. */
 gemm_status_t kselect_wait_selftest(int64_t limit_ns, int32_t* waited_out, void* stream);
+
+/* Test hooks of the FP32 products on the tensor cores (no paper counterpart).
+ * kselect_f32tc_selftest runs one, whatever gemm() would choose, with 128 x bn
+ * tiles (bn 64 or 128) or 256 x 256 tiles on CTA pairs (bn 256) and K divided
+ * into up to `splits` (1..16) ranges whose partial products a second kernel
+ * sums; the other arguments are gemm_strided_batched's.  K = 0 is UNSUPPORTED.
+ * kselect_f32tc_choice returns the bn that a handle call uses instead of SIMT
+ * config `config_id` (0: it runs the config), and the split factor, for these
+ * sizes; `aligned` says whether every row allows 16-byte access.  Needs a GPU
+ * for the occupancy query.  Negative gemm_status_t on error. */
+gemm_status_t kselect_f32tc_selftest(int32_t bn, int32_t splits, char transA, char transB, int64_t M, int64_t N,
+                                     int64_t K, float alpha, const float* A_dev, int64_t lda, int64_t strideA,
+                                     const float* B_dev, int64_t ldb, int64_t strideB, float beta, float* C_dev,
+                                     int64_t ldc, int64_t strideC, int64_t batch, void* stream);
+int32_t kselect_f32tc_choice(int32_t config_id, int64_t M, int64_t N, int64_t K, int64_t batch, int32_t transA,
+                             int32_t aligned, int32_t* splits);
 
 /* Fills a (batch, rows, ld) float array with uniform[lo, hi) values from a
  * counter-based hash of (seed, element index); padding columns get `pad`.

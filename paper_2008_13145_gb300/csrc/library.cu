@@ -335,6 +335,159 @@ static gemm_status_t launch_split(int base, const GemmArgs& a, int splits, int k
   return GEMM_OK;
 }
 
+// ------------------------------------------------------------------ FP32 on the tensor cores (f32tc.cu)
+cudaError_t f32tc_launch(int bn, const GemmArgs& g, int splits, int kchunk, int sms, int* status, cudaStream_t s);
+int* tc_status_word();
+int* tc_status_word_if_ready();
+
+struct F32tcPlan {
+  int bn;  // 64 or 128: 128 x bn tiles; 256: 256 x 256 tiles on CTA pairs
+  int splits, kchunk;
+};
+
+// Time models of the two ways to run an FP32 product, in microseconds, fitted
+// to 500 shapes of the tuning grid's ranges (every tile width and up to eight
+// split factors each, aligned and odd rows, on GB300).
+//
+// Tensor cores: a launch, then per round of items (tiles x splits over the
+// CTAs or CTA pairs) its K chunks of 32 and its stores; rows that allow no
+// 16-byte access cost more; splits add the reduction.  5 to 95 % of the
+// fitted times lie within 0.80 .. 1.16 of the measured ones.
+struct F32tcCost {
+  int bn;
+  double call, chunk, chunk_odd_k, chunk_odd_m, item, item_odd, reduce, reduce_mb;
+};
+constexpr F32tcCost kF32tcCost[3] = {{64, 6.0, 0.71, 0.04, 0.10, 1.1, 0.4, 1.9, 0.07},
+                                     {128, 5.1, 1.03, 0.02, 0.14, 2.6, 0.9, 0.8, 0.12},
+                                     {256, 6.4, 1.43, 0.01, 0.11, 3.9, 1.2, 0.4, 0.20}};
+// SIMT (and split-K): a launch, per wave the K range plus half a K-step at the
+// full-wave rate, and the reduction; 5 to 95 % within 0.79 .. 1.21.
+constexpr double kSimtCall = 6.2, kSimtK = 0.95, kSimtStep = 0.49, kSimtSplit = 3.1, kSimtReduceMb = 0.023;
+// The tensor cores run what they are expected to win by this factor, and only
+// products that keep the GPU busier than a call's host work does.  With these
+// three the worst of the 500 lost 13 % (21 against 24 us), two more lost 8 and
+// 9 %, and the geometric mean gain over all is 1.27 of the 1.34 that the faster
+// of the two would give; with neither minimum and a factor of 1 the worst lost
+// 40 %, and 256 x 256 x 256 took 20 us a call, split in four, against 14.
+constexpr double kF32tcMargin = 1.15;
+constexpr double kF32tcMinFlops = 2e8;
+constexpr double kF32tcMinSimtUs = 16.0;
+constexpr double kF32tcSplitHostUs = 3.0;  // host work of a second launch and its workspace
+// Below two K chunks the SIMT tiles, whose stores overlap other CTAs' loads,
+// stay ahead wherever they were measured to within the model's error.
+constexpr int kF32tcMinK = 64;
+constexpr int kF32tcChunk = 32;
+
+static double f32tc_cost(const F32tcCost& c, const GemmArgs& a, int64_t tiles, int64_t kc, int splits, int units) {
+  const int64_t rounds = ceil_div(tiles * splits, units);
+  const double odd = a.vecA && a.vecB ? 0.0 : a.transA ? c.chunk_odd_m : c.chunk_odd_k;
+  double us = c.call + (double)rounds * ((double)kc * (c.chunk + odd) + c.item + (a.vecC ? 0.0 : c.item_odd));
+  if (splits > 1) us += kF32tcSplitHostUs + c.reduce + c.reduce_mb * (splits + 2.0) * a.batch * a.M * (double)a.N * 4e-6;
+  return us;
+}
+
+// Mean squared relative error of both against the exact product, in units of
+// 2^-48, for non-negative operands, where rounding errors add up worst (uniform
+// [0, 1) data at K 64 .. 4096, each split factor: fits within 15 %).  The SIMT
+// chain rounds once per K; the tensor cores' chunk sums carry a truncation of
+// 0.86 2^-24 on average, and a rounding per chunk.  A plan is considered only
+// where it is the more exact one; on signed data it then is by a factor of 1.4
+// to 7 (all of the 500 shapes).
+static double f32tc_error(double K, int S) { return 1.13 + 0.0015 * K / ((double)S * S) + (S > 1 ? 0.04 * S : 0.0); }
+static double simt_error(double K, int S) { return 0.05 * K / ((double)S * S) + (S > 1 ? 0.07 * S : 0.0); }
+
+// *splits receives the split factor the model assumes.
+static double simt_cost(int id, const GemmArgs& a, int dev, int sms, int* splits) {
+  const int base = id >= kSplitBase ? id - kSplitBase : id;
+  const SimtParams P = simt_params(base);
+  const int BM = P.wy * P.tm, BN = P.wx * P.tn;
+  int occ = split_eligible(base) ? occupancy_of(base, dev) : 0;
+  if (occ < 1) occ = 4;
+  int kc = a.K, S = 1;
+  if (id >= kSplitBase) S = choose_split(a.M, a.N, a.K, a.batch, BM, BN, P.bk, occ, sms, &kc);
+  const double cap = (double)occ * sms;
+  const double waves = (double)(ceil_div(a.M, BM) * ceil_div(a.N, BN)) * a.batch * S / cap;
+  const double w = waves <= 1.0 ? 1.0 : 0.5 * (waves + std::ceil(waves));
+  const double unit = 2e6 * BM * BN * cap / kSplitFlopRate;  // one K element of a full wave
+  double us = kSimtCall + w * unit * (kSimtK * a.K / S + kSimtStep * P.bk);
+  *splits = S;
+  if (S > 1) us += kSimtSplit + kSimtReduceMb * (S + 2.0) * a.batch * a.M * (double)a.N * 4e-6;
+  return us;
+}
+
+// Whether an FP32 request for which SIMT kernel `id` was selected runs on the
+// tensor cores, and how.  Split factors tried: those that fill one round and two
+// rounds of CTAs, since the model's cost falls with the K range of an item and
+// rises with the rounds (this runs on every call, so it stays short).
+static bool f32tc_plan(int id, const GemmArgs& a, int dev, int sms, F32tcPlan* plan) {
+  if (a.K < kF32tcMinK || sms < 2) return false;
+  const double outputs = (double)a.M * (double)a.N * (double)a.batch;
+  if (outputs > 1e12) return false;  // keeps the tile counts small
+  if (2.0 * outputs * a.K < kF32tcMinFlops) return false;
+  int simt_splits = 1;
+  double best = simt_cost(id, a, dev, sms, &simt_splits);
+  if (best < kF32tcMinSimtUs) return false;
+  best /= kF32tcMargin;
+  const double error = 0.9 * simt_error(a.K, simt_splits);
+  bool found = false;
+  const int nk = (a.K + kF32tcChunk - 1) / kF32tcChunk;
+  const int64_t slab = (int64_t)a.batch * a.M * (((int64_t)a.N + 7) / 8 * 8) * 4;
+  for (const F32tcCost& c : kF32tcCost) {
+    const int bm = c.bn == 256 ? 256 : 128, units = c.bn == 256 ? sms / 2 : sms;
+    const int64_t tiles = ceil_div(a.M, bm) * ceil_div(a.N, c.bn) * a.batch;
+    int last = 0;
+    for (int rounds = 0; rounds <= 2; ++rounds) {
+      int S = rounds == 0 ? 1 : (int)std::min<int64_t>(rounds * units / tiles, std::min(kSplitMaxFactor, nk / 2));
+      if (S <= last) continue;
+      const int kc = (nk + S - 1) / S;
+      S = (nk + kc - 1) / kc;
+      if (S <= last) continue;
+      last = S;
+      if (S > 1 && S * slab > kSplitWorkspaceMax) break;
+      if (f32tc_error(a.K, S) > error) continue;
+      const double us = f32tc_cost(c, a, tiles, kc, S, units);
+      if (us < best) {
+        best = us;
+        found = true;
+        *plan = F32tcPlan{c.bn, S, kc * kF32tcChunk};
+      }
+    }
+  }
+  return found;
+}
+
+static gemm_status_t f32tc_run(const F32tcPlan& plan, const GemmArgs& a, int sms, int* status, cudaStream_t s) {
+  const int bn = plan.bn, splits = plan.splits, kchunk = plan.kchunk;
+  cudaError_t e;
+  if (splits <= 1) {
+    e = f32tc_launch(bn, a, 1, a.K, sms, status, s);
+    if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
+    return GEMM_OK;
+  }
+  const int64_t ldw = ((int64_t)a.N + 7) / 8 * 8;
+  void* w = nullptr;
+  e = split_alloc(&w, (size_t)splits * a.batch * a.M * ldw * sizeof(float), s);
+  if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
+  GemmArgs p = a;
+  p.alpha = 1.f;
+  p.beta = 0.f;
+  p.C = static_cast<float*>(w);
+  p.ldc = ldw;
+  p.strideC = ldw * a.M;
+  p.vecC = 1;
+  e = f32tc_launch(bn, p, splits, kchunk, sms, status, s);
+  if (e == cudaSuccess) {
+    const int64_t total = (int64_t)a.batch * a.M * ((a.N + 3) / 4);
+    const int grid = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
+    e = launch_pdl(split_reduce_kernel, dim3(grid), dim3(256), 0, s, nullptr, 0, static_cast<const float*>(w), ldw,
+                   splits, a.M, a.N, a.batch, a.alpha, a.beta, a.C, a.ldc, a.strideC, a.vecC, a);
+  }
+  cudaError_t ef = cudaFreeAsync(w, s);
+  if (e == cudaSuccess) e = ef;
+  if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
+  return GEMM_OK;
+}
+
 // C = beta * C, for K == 0 (the product term vanishes).
 __global__ void scale_c_kernel(float* C, int64_t ldc, int64_t strideC, int M, int N, float beta) {
   const int64_t total = (int64_t)M * N;
@@ -378,6 +531,27 @@ static gemm_status_t launch_config(int id, const GemmArgs& a, cudaStream_t s) {
   }
   if (fam > 0) return tc_launch(id, a, s);
   return GEMM_ERR_NO_KERNEL;
+}
+
+// Runs the kernel a handle selected.  A SIMT choice is run on the tensor cores
+// at FP32 accuracy (f32tc.cu: closer to the exact product than the SIMT kernels'
+// FMA chains) where that is expected to be faster.  The device's first
+// tensor-core call allocates, so under stream capture it stays with the choice.
+static gemm_status_t launch_selected(int id, const GemmArgs& a, cudaStream_t s) {
+  if (family_of(id) != GEMM_PREC_F32) return launch_config(id, a, s);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return launch_config(id, a, s);
+  const int sms = sm_count_of(dev);
+  F32tcPlan plan;
+  if (!f32tc_plan(id, a, dev, sms, &plan)) return launch_config(id, a, s);
+  int* status = tc_status_word_if_ready();
+  if (!status) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+      return launch_config(id, a, s);
+    if (!(status = tc_status_word())) return launch_config(id, a, s);
+  }
+  return f32tc_run(plan, a, sms, status, s);
 }
 
 static int elem_bytes_of(int id) { return family_of(id) == GEMM_PREC_BF16 ? 2 : 4; }
@@ -638,8 +812,12 @@ gemm_status_t gemm_strided_batched(gemm_handle_t h, char transA, char transB, in
   if (!h) return GEMM_ERR_INVALID_ARG;
   const int32_t id = select_kernel(h, M, N, K, batch);
   if (id < 0) return (gemm_status_t)id;
-  return gemm_strided_batched_with_config(id, transA, transB, M, N, K, alpha, A, lda, strideA, B, ldb, strideB, beta,
-                                          C, ldc, strideC, batch, stream);
+  GemmArgs a;
+  bool noop = false;
+  gemm_status_t st = strided_args(id, transA, transB, M, N, K, alpha, A, lda, strideA, B, ldb, strideB, beta, C, ldc,
+                                  strideC, batch, &a, &noop);
+  if (st != GEMM_OK || noop) return st;
+  return launch_selected(id, a, static_cast<cudaStream_t>(stream));
 }
 
 gemm_status_t gemm_with_config(int32_t id, char transA, char transB, int64_t M, int64_t N, int64_t K,
@@ -688,7 +866,51 @@ gemm_status_t gemm(gemm_handle_t h, char transA, char transB, int64_t M, int64_t
   if (!h) return GEMM_ERR_INVALID_ARG;
   const int32_t id = select_kernel(h, M, N, K, batch);
   if (id < 0) return (gemm_status_t)id;
-  return gemm_with_config(id, transA, transB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, batch, stream);
+  GemmArgs a;
+  bool noop = false;
+  gemm_status_t st = make_args(transA, transB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, batch,
+                               elem_bytes_of(id), &a, &noop);
+  if (st != GEMM_OK || noop) return st;
+  return launch_selected(id, a, static_cast<cudaStream_t>(stream));
+}
+
+gemm_status_t kselect_f32tc_selftest(int32_t bn, int32_t splits, char transA, char transB, int64_t M, int64_t N,
+                                     int64_t K, float alpha, const float* A, int64_t lda, int64_t strideA,
+                                     const float* B, int64_t ldb, int64_t strideB, float beta, float* C, int64_t ldc,
+                                     int64_t strideC, int64_t batch, void* stream) {
+  if ((bn != 64 && bn != 128 && bn != 256) || splits < 1 || splits > kSplitMaxFactor) return GEMM_ERR_INVALID_ARG;
+  GemmArgs a;
+  bool noop = false;
+  gemm_status_t st = strided_args(0, transA, transB, M, N, K, alpha, A, lda, strideA, B, ldb, strideB, beta, C, ldc,
+                                  strideC, batch, &a, &noop);
+  if (st != GEMM_OK || noop) return st;
+  if (K == 0 || (double)M * (double)N * (double)batch > 1e12) return GEMM_ERR_UNSUPPORTED;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  int* status = e == cudaSuccess ? tc_status_word() : nullptr;
+  if (!status) { set_last_cuda_error(e != cudaSuccess ? e : cudaGetLastError()); return GEMM_ERR_CUDA; }
+  const int64_t kc = ceil_div(ceil_div(K, splits), kF32tcChunk) * kF32tcChunk;
+  const F32tcPlan plan{bn, (int)ceil_div(K, kc), (int)kc};
+  return f32tc_run(plan, a, sm_count_of(dev), status, static_cast<cudaStream_t>(stream));
+}
+
+int32_t kselect_f32tc_choice(int32_t id, int64_t M, int64_t N, int64_t K, int64_t batch, int32_t transA,
+                             int32_t aligned, int32_t* splits) {
+  if (!splits || family_of(id) != GEMM_PREC_F32) return GEMM_ERR_INVALID_ARG;
+  GemmArgs a;
+  bool noop = false;
+  float dummy = 0.f;
+  gemm_status_t st = make_args(transA ? 'T' : 'N', 'N', M, N, K, 1.f, &dummy, std::max<int64_t>(M, K), &dummy,
+                               std::max<int64_t>(N, 1), 0.f, &dummy, std::max<int64_t>(N, 1), batch, 4, &a, &noop);
+  if (st != GEMM_OK) return st;
+  *splits = 1;
+  a.vecA = a.vecB = a.vecC = aligned != 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return GEMM_ERR_CUDA;
+  F32tcPlan plan;
+  if (noop || !f32tc_plan(id, a, dev, sm_count_of(dev), &plan)) return 0;
+  *splits = plan.splits;
+  return plan.bn;
 }
 
 gemm_status_t gemm_host(gemm_handle_t h, char transA, char transB, int64_t M, int64_t N, int64_t K, float alpha,
@@ -714,7 +936,7 @@ gemm_status_t gemm_host(gemm_handle_t h, char transA, char transB, int64_t M, in
   }
   if (e == cudaSuccess && beta != 0.f) e = cudaMemcpyAsync(C_dev, C_host, bytesC, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
-  st = launch_config(id, a, s);
+  st = launch_selected(id, a, s);
   if (st != GEMM_OK) return st;
   e = cudaMemcpyAsync(C_host, C_dev, bytesC, cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
@@ -785,7 +1007,7 @@ gemm_status_t gemm_host_pipeline(gemm_handle_t h, int32_t count, const gemm_host
     if (e == cudaSuccess) e = cudaEventRecord(ev[1 + 2 * i], up);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev[1 + 2 * i], 0);
     if (e != cudaSuccess) break;
-    st = launch_config(ids[i], a, s);
+    st = launch_selected(ids[i], a, s);
     if (st != GEMM_OK) break;
     e = cudaEventRecord(ev[2 + 2 * i], s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(down, ev[2 + 2 * i], 0);

@@ -483,6 +483,9 @@ OperandPlan plan_operand(const TcConfig& c, const void* ptr, int64_t ld, int64_t
 
 }  // namespace
 
+int* tc_status_word() { return status_word(); }
+int* tc_status_word_if_ready() { return status_word_if_ready(); }
+
 bool tc_config_valid(int id) {
   TcConfig c;
   return decode(id, &c);
