@@ -125,6 +125,13 @@ gemm_status_t tc_params(int id, int32_t out[8]);
 
 void set_last_cuda_error(cudaError_t e);
 
+// Stream-ordered scratch of one call, freed with cudaFreeAsync on the same
+// stream (library.cu).
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+// Counts handles; with the last one gone the scratch pools' idle memory goes back to the device.
+void scratch_add_handle();
+void scratch_drop_handle();
+
 }  // namespace ks
 
 // The library handle: an immutable deployment plus a per-device cache of the
@@ -155,11 +162,15 @@ struct kselect_library {
   char* dev_ws[64] = {nullptr};
   int64_t dev_ws_bytes[64] = {0};
   std::vector<char*> retired_ws;
+  kselect_library() { ks::scratch_add_handle(); }
+  kselect_library(const kselect_library&) = delete;
+  kselect_library& operator=(const kselect_library&) = delete;
   ~kselect_library() {
     for (float* p : dev_mlp)
       if (p) cudaFree(p);
     for (char* p : dev_ws)
       if (p) cudaFree(p);
     for (char* p : retired_ws) cudaFree(p);
+    ks::scratch_drop_handle();
   }
 };

@@ -7,8 +7,16 @@
 // tensor core truncates each addition into its accumulator, so a K chunk of 32
 // is all that one accumulator sums: the small products first, then the two
 // steps of p0 q0.  The chunk sums are then added in FP32, rounded to nearest,
-// in registers.  The result is closer to the exact product than a chain of
-// FP32 FMAs over K (measured against 64 bits, see f32tc_plan).
+// in registers.  Relative error against 64 bits at 4096 x 4096 x 4096, uniform
+// [-1, 1): 2.1e-7 (a chain of FP32 FMAs over K: 1.15e-6); f32tc_plan uses the
+// kernel only where it is the more exact of the two.
+//
+// Bound: six 16-bit products, 315 TFLOP/s of the measured BF16 rate; the FP32
+// pipe's peak is 80.  4096 x 4096 x 4096: 625 us, 220 TFLOP/s (A B^T 590 us, 233;
+// the last of four rounds of 256 x 256 tiles is a third full: 277 at 4864 x 4096 x
+// 4096) against 2,520 us for the SIMT kernel.  What holds it is the converting
+// warps' chain of latencies (load, split, store, fence per chunk), then
+// shared-memory bandwidth: the MMAs of 128-wide tiles alone read 128 bytes a clock.
 //
 // A split that is not exact (infinities, NaN, magnitudes whose low bits fall
 // below BF16's range, values that round past the largest BF16) is seen while

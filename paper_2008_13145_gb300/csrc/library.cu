@@ -266,32 +266,55 @@ __global__ void split_reduce_kernel(const float* __restrict__ W, int64_t ldw, in
   }
 }
 
-// Stream-ordered workspace for the partial tiles: a per-device pool that keeps
-// its memory between calls; under stream capture the default pool is used so
-// that the allocation becomes a graph node.
-static cudaError_t split_alloc(void** p, size_t bytes, cudaStream_t s) {
+// Stream-ordered scratch (split-K partials, pre-pass operands, training
+// workspaces) comes from one pool per device that keeps up to kScratchKeep of
+// idle memory across synchronisations: CUDA's default pool keeps none, so every
+// call after a synchronisation mapped its scratch anew (220 us for an x3 product
+// of 29 us).  Idle memory goes back when the last handle is destroyed.  Pools
+// are made once and are safe with several threads and streams; under stream
+// capture the default pool is used, so that the allocation becomes a graph node.
+constexpr uint64_t kScratchKeep = 2ull << 30;
+static std::mutex g_scratch_mu;
+static std::atomic<cudaMemPool_t> g_scratch_pools[64];
+static int g_scratch_handles = 0;
+
+void scratch_add_handle() {
+  std::lock_guard<std::mutex> lk(g_scratch_mu);
+  ++g_scratch_handles;
+}
+
+void scratch_drop_handle() {
+  std::lock_guard<std::mutex> lk(g_scratch_mu);
+  if (--g_scratch_handles > 0) return;
+  // A handle may go while some thread captures a stream: trimming is no part of that capture.
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  for (auto& p : g_scratch_pools)
+    if (cudaMemPool_t pool = p.load(std::memory_order_relaxed)) cudaMemPoolTrimTo(pool, 0);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaStreamIsCapturing(s, &cs);
   if (e != cudaSuccess) return e;
   if (cs != cudaStreamCaptureStatusNone) return cudaMallocAsync(p, bytes, s);
-  static std::mutex mu;
-  static cudaMemPool_t pools[64] = {};
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  cudaMemPool_t pool;
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    if (!pools[dev]) {
+  cudaMemPool_t pool = g_scratch_pools[dev].load(std::memory_order_acquire);
+  if (!pool) {
+    std::lock_guard<std::mutex> lk(g_scratch_mu);
+    if (!(pool = g_scratch_pools[dev].load(std::memory_order_relaxed))) {
       cudaMemPoolProps props = {};
       props.allocType = cudaMemAllocationTypePinned;
       props.location.type = cudaMemLocationTypeDevice;
       props.location.id = dev;
-      if ((e = cudaMemPoolCreate(&pools[dev], &props)) != cudaSuccess) { pools[dev] = nullptr; return e; }
-      uint64_t keep = UINT64_MAX;
-      cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+      if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
+      uint64_t keep = kScratchKeep;
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+      g_scratch_pools[dev].store(pool, std::memory_order_release);
     }
-    pool = pools[dev];
   }
   return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
@@ -302,7 +325,7 @@ static gemm_status_t launch_split(int base, const GemmArgs& a, int splits, int k
   const int64_t ldw = ((int64_t)a.N + 3) / 4 * 4;
   const size_t bytes = (size_t)splits * a.batch * a.M * ldw * sizeof(float);
   void* w = nullptr;
-  cudaError_t e = split_alloc(&w, bytes, s);
+  cudaError_t e = scratch_alloc(&w, bytes, s);
   if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
   GemmArgs p = a;
   p.alpha = 1.f;
@@ -466,7 +489,7 @@ static gemm_status_t f32tc_run(const F32tcPlan& plan, const GemmArgs& a, int sms
   }
   const int64_t ldw = ((int64_t)a.N + 7) / 8 * 8;
   void* w = nullptr;
-  e = split_alloc(&w, (size_t)splits * a.batch * a.M * ldw * sizeof(float), s);
+  e = scratch_alloc(&w, (size_t)splits * a.batch * a.M * ldw * sizeof(float), s);
   if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
   GemmArgs p = a;
   p.alpha = 1.f;

@@ -296,7 +296,7 @@ struct Workspace {
 
 cudaError_t ws_alloc(int nblocks, cudaStream_t s, Workspace* w) {
   const size_t bytes = sizeof(float) * ((size_t)nblocks * NP + nblocks + 1 + NP + 1) + sizeof(int) + 6 * 256;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&w->base), bytes, s);
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&w->base), bytes, s);
   if (e != cudaSuccess) return e;
   char* p = w->base;
   auto carve = [&](size_t nb) {

@@ -516,7 +516,7 @@ gemm_status_t tc_launch(int id, const GemmArgs& g, cudaStream_t s) {
   OperandPlan pb = plan_operand(c, g.B, g.ldb, g.strideB, g.transB != 0, g.N, g.K, g.batch, b_ext);
   char* scratch = nullptr;
   if (pa.bytes + pb.bytes > 0) {
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), pa.bytes + pb.bytes + 256, s);
+    cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&scratch), pa.bytes + pb.bytes + 256, s);
     if (e != cudaSuccess) return fail(e);
   }
   const void* Aop = pa.direct ? g.A : scratch;
