@@ -382,7 +382,7 @@ cudaError_t launch_kernel(const CUtensorMap& ma, const CUtensorMap& mb, const tc
     const int regs = (fa.numRegs + 7) / 8 * 8;
     const int per_cta = (int)fa.sharedSizeBytes + reserved;
     const int occ_smem = smem_sm / (Cfg::SMEM_BYTES + per_cta);
-    int occ = std::min(occ_smem, regs_sm / (regs * tc::kThreads));
+    int occ = std::min(occ_smem, regs_sm / (regs * Cfg::THREADS));
     occ = std::max(1, std::min(occ, 512 / Cfg::TMEM_COLS));  // every resident CTA must fit in TMEM
     // Where shared memory alone would let more CTAs onto an SM than TMEM or the
     // registers hold (BN 128 and BN 256 with two stages), ask for enough of it that
@@ -399,7 +399,7 @@ cudaError_t launch_kernel(const CUtensorMap& ma, const CUtensorMap& mb, const tc
     __atomic_fetch_or(&done_mask, bit, __ATOMIC_ACQ_REL);
   }
   const int ctas = std::min(a.num_tiles, slots_cache[dev & 63]);
-  return launch_pdl(kern, dim3((unsigned)ctas, 1, 1), dim3(tc::kThreads, 1, 1), (size_t)dyn_cache[dev & 63], s,
+  return launch_pdl(kern, dim3((unsigned)ctas, 1, 1), dim3(Cfg::THREADS, 1, 1), (size_t)dyn_cache[dev & 63], s,
                     nullptr, 0, ma, mb, a, g);
 }
 
@@ -430,6 +430,12 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 gemm_status_t fail(cudaError_t e) {
   set_last_cuda_error(e);
   return GEMM_ERR_CUDA;
+}
+
+// Width of the accesses that every row of C allows: 2 = 32 bytes, 1 = 16, 0 = 4.
+int vec_of(const float* C, int64_t ldc, int64_t stride) {
+  if ((uintptr_t)C % 32 == 0 && ldc % 8 == 0 && stride % 8 == 0) return 2;
+  return (uintptr_t)C % 16 == 0 && ldc % 4 == 0 && stride % 4 == 0;
 }
 
 // How one operand reaches the kernel: in place, or through a rewrite job.
@@ -558,7 +564,7 @@ gemm_status_t tc_launch(int id, const GemmArgs& g, cudaStream_t s) {
     a.raster = 2;
     a.group_m = std::max(1, std::min(a.tiles_m, kRasterGroup));
     a.alpha = g.alpha; a.beta = g.beta;
-    a.C = g.C; a.ldc = g.ldc; a.strideC = g.strideC; a.vecC = g.vecC;
+    a.C = g.C; a.ldc = g.ldc; a.strideC = g.strideC; a.vecC = vec_of(g.C, g.ldc, g.batch == 1 ? 0 : g.strideC);
     a.a_mn = pa.mn; a.b_mn = pb.mn;
     a.seg_blocks = x3 ? (int)(round_up(g.K, kSplitSeg) / 64) : 0;
     a.seg_map = x3 ? sp.seg_map : 0;
@@ -705,7 +711,7 @@ gemm_status_t group_encode(const GroupBuild& b, const gemm_problem_t* probs, cha
     d.tiles_m = row_tiles(q.M);
     d.tiles_n = (int)((q.N + c.bn - 1) / c.bn);
     d.tile_start = tile_start;
-    d.vecC = ((uintptr_t)q.C % 16 == 0) && (q.ldc % 4 == 0);
+    d.vecC = vec_of(q.C, q.ldc, 0);
     d.a_mn = pa.mn;
     d.b_mn = pb.mn;
     d.seg_blocks = x3 ? (int)(round_up(q.K, kSplitSeg) / 64) : 0;

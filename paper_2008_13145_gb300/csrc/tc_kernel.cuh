@@ -5,12 +5,12 @@
 // instead be MN-contiguous (A stored K x M, B stored K x N), in which case it
 // is staged as MN-major tiles and the MMA reads it transposed.  Tiles of
 // 128 x BN outputs are distributed over persistent CTAs; each CTA runs
-//   warp 4      : TMA producer (one elected lane) filling a STAGES-deep ring
-//                 of 128-byte-swizzled A/B slices, 128 bytes of K per slice;
-//   warp 5      : TMEM allocator and MMA issuer (one elected lane), 4
-//                 tcgen05.mma per slice into an FP32 accumulator in TMEM;
 //   warps 0..3  : epilogue, tcgen05.ld of their 32-lane quadrant, alpha/beta,
-//                 vector stores of C.
+//                 vector stores of C (BN 256: warps 0..7, two per quadrant);
+//   next warp   : TMA producer (one elected lane) filling a STAGES-deep ring
+//                 of 128-byte-swizzled A/B slices, 128 bytes of K per slice;
+//   last warp   : TMEM allocator and MMA issuer (one elected lane), 4
+//                 tcgen05.mma per slice into an FP32 accumulator in TMEM.
 // Two TMEM accumulators (2 x BN columns) let the epilogue of tile i overlap
 // the MMAs of tile i+1.  With GROUPED, the launch covers an uneven group of
 // problems: the global tile index is mapped to (problem, tile) by binary
@@ -32,7 +32,7 @@ struct TcArgs {
   float alpha, beta;
   float* C;
   int64_t ldc, strideC;
-  int vecC;
+  int vecC;  // C takes 16-byte accesses (1) or 32-byte ones (2)
   int a_mn, b_mn;  // operand staged MN-major
   // Split-BF16 products: each operand holds nseg segments of seg_blocks
   // K-slices (its BF16 split parts, largest first) and segment g of the K'
@@ -60,7 +60,6 @@ struct GroupArgs {
   int count;  // problems; descs[i].tile_start is ascending
 };
 
-constexpr int kThreads = 192;
 constexpr int kBM = 128;
 
 template <int BN, int STAGES, bool TF32>
@@ -72,8 +71,13 @@ struct TcCfg {
   static constexpr int B_BYTES = BN * 128;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int TMEM_COLS = 2 * BN;     // 128, 256 or 512: power of two >= 32
-  // Epilogue staging: 32 rows x 16 FP32 columns per epilogue warp.
-  static constexpr int EPI_BYTES = 4 * 32 * 16 * 4;
+  // Epilogue warps: two per TMEM lane quadrant, each with half of the columns,
+  // where one CTA has the SM to itself; one where two or three share it.
+  static constexpr int EPI_WARPS = BN == 256 ? 8 : 4;
+  static constexpr int THREADS = 32 * (EPI_WARPS + 2);
+  // Epilogue staging: 32 rows x STORE_COLS FP32 columns per epilogue warp.
+  static constexpr int STORE_COLS = BN == 256 ? 32 : 16;
+  static constexpr int EPI_BYTES = EPI_WARPS * 32 * STORE_COLS * 4;
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024;
   // MN-major staging: one TMA box is MN_BOX MN elements (a 128-byte row) by
   // BK K rows; the boxes of a slice lie MN-block after MN-block.  The swizzle
@@ -149,57 +153,100 @@ __device__ __forceinline__ TileLoc locate(const TcArgs& p, const GroupArgs& g, c
 
 // Stores one 32 x 32 chunk of C (rows row0 + lane of this warp's 32-row
 // quadrant, columns n0 .. n0 + 31) from the registers of tcgen05.ld, where
-// lane t holds row t.  Each 16-column half goes through this warp's 2 KB
-// staging buffer (64-byte rows; the 16-byte piece q of row t sits at
-// (t & 1) * 4 + (q ^ ((t >> 1) & 3)) within its 128-byte bank line, so both
-// passes are free of bank conflicts) and is written back eight rows per
-// instruction, each row a contiguous 64-byte run of C; beta != 0 reads C the
-// same way.
+// lane t holds row t.  When every row of C starts on 32 bytes, each lane writes
+// whole 32-byte sectors of its own row.  Otherwise SC (16 or 32) columns at a
+// time go through this warp's staging buffer (the 16-byte piece q of row t sits
+// at q ^ t, or q ^ (t / 2) within 64-byte rows, so both passes are free of bank
+// conflicts) and leave as contiguous runs of a row: 16 bytes a lane where C
+// allows it, else 4.  beta != 0 reads C the same way.  Together with the second
+// epilogue warp per quadrant this took f32mix 1733 x 912 x 1408 x 2 from 77 to 48
+// us, an uneven BF16 group of 256 from 509 to 443 and, with rows of 637 floats,
+// BF16 2185 x 637 x 95 x 16 from 87 to 63 (its lanes wrote 4 bytes every 16).
+template <int SC>
 __device__ __forceinline__ void store_chunk32(const TileLoc& p, float* cbase, int row0, int n0, float* stage,
                                               const uint32_t (&r)[32], int lane) {
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  if (p.vecC == 2 && n0 + 32 <= p.N) {
+    if (row0 + lane >= p.M) return;
+    float* dst = cbase + (int64_t)(row0 + lane) * p.ldc + n0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int c = 16 * h + 4 * q;
+      float o[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[e] = p.alpha * __uint_as_float(r[8 * q + e]);
+      if (p.beta != 0.f) {
+        const float4 c0 = *reinterpret_cast<const float4*>(dst + 8 * q);
+        const float4 c1 = *reinterpret_cast<const float4*>(dst + 8 * q + 4);
+        o[0] = fmaf(p.beta, c0.x, o[0]); o[1] = fmaf(p.beta, c0.y, o[1]);
+        o[2] = fmaf(p.beta, c0.z, o[2]); o[3] = fmaf(p.beta, c0.w, o[3]);
+        o[4] = fmaf(p.beta, c1.x, o[4]); o[5] = fmaf(p.beta, c1.y, o[5]);
+        o[6] = fmaf(p.beta, c1.z, o[6]); o[7] = fmaf(p.beta, c1.w, o[7]);
+      }
+      asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 8 * q), "f"(o[0]),
+                   "f"(o[1]), "f"(o[2]), "f"(o[3]), "f"(o[4]), "f"(o[5]), "f"(o[6]), "f"(o[7])
+                   : "memory");
+    }
+    return;
+  }
+  constexpr int P = SC / 4;              // 16-byte pieces of a staged row
+  constexpr int SH = SC == 16 ? 1 : 0;   // rows that share a 128-byte line, as a shift
+#pragma unroll
+  for (int h = 0; h < 32 / SC; ++h) {
+#pragma unroll
+    for (int q = 0; q < P; ++q) {
+      const int c = SC * h + 4 * q;
       const float4 v = make_float4(__uint_as_float(r[c]), __uint_as_float(r[c + 1]), __uint_as_float(r[c + 2]),
                                    __uint_as_float(r[c + 3]));
-      *reinterpret_cast<float4*>(stage + lane * 16 + ((q ^ ((lane >> 1) & 3)) << 2)) = v;
+      *reinterpret_cast<float4*>(stage + lane * SC + ((q ^ ((lane >> SH) & (P - 1))) << 2)) = v;
     }
     __syncwarp();
-    const int q = lane & 3, n = n0 + 16 * h + 4 * q;
+    if (p.vecC) {
+      const int q = lane & (P - 1), n = n0 + SC * h + 4 * q;
 #pragma unroll 2
-    for (int i = 0; i < 4; ++i) {
-      const int rr = 8 * i + (lane >> 2), row = row0 + rr;
-      const float4 v = *reinterpret_cast<const float4*>(stage + rr * 16 + ((q ^ ((rr >> 1) & 3)) << 2));
-      if (row >= p.M || n >= p.N) continue;
-      float* crow = cbase + (int64_t)row * p.ldc;
-      if (p.vecC && n + 3 < p.N) {
-        float4 o = make_float4(p.alpha * v.x, p.alpha * v.y, p.alpha * v.z, p.alpha * v.w);
-        if (p.beta != 0.f) {
-          const float4 c = *reinterpret_cast<const float4*>(crow + n);
-          o.x = fmaf(p.beta, c.x, o.x); o.y = fmaf(p.beta, c.y, o.y);
-          o.z = fmaf(p.beta, c.z, o.z); o.w = fmaf(p.beta, c.w, o.w);
-        }
-        *reinterpret_cast<float4*>(crow + n) = o;
-      } else {
-        const float e4[4] = {v.x, v.y, v.z, v.w};
+      for (int i = 0; i < P; ++i) {
+        const int rr = (32 / P) * i + lane / P, row = row0 + rr;
+        const float4 v = *reinterpret_cast<const float4*>(stage + rr * SC + ((q ^ ((rr >> SH) & (P - 1))) << 2));
+        if (row >= p.M || n >= p.N) continue;
+        float* crow = cbase + (int64_t)row * p.ldc;
+        if (n + 3 < p.N) {
+          float4 o = make_float4(p.alpha * v.x, p.alpha * v.y, p.alpha * v.z, p.alpha * v.w);
+          if (p.beta != 0.f) {
+            const float4 c = *reinterpret_cast<const float4*>(crow + n);
+            o.x = fmaf(p.beta, c.x, o.x); o.y = fmaf(p.beta, c.y, o.y);
+            o.z = fmaf(p.beta, c.z, o.z); o.w = fmaf(p.beta, c.w, o.w);
+          }
+          *reinterpret_cast<float4*>(crow + n) = o;
+        } else {
+          const float e4[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          if (n + e < p.N) {
-            float o = p.alpha * e4[e];
-            if (p.beta != 0.f) o = fmaf(p.beta, crow[n + e], o);
-            crow[n + e] = o;
+          for (int e = 0; e < 4; ++e) {
+            if (n + e < p.N) {
+              float o = p.alpha * e4[e];
+              if (p.beta != 0.f) o = fmaf(p.beta, crow[n + e], o);
+              crow[n + e] = o;
+            }
           }
         }
       }
+    } else {
+      const int c = lane & (SC - 1), n = n0 + SC * h + c;
+#pragma unroll 4
+      for (int i = 0; i < SC; ++i) {
+        const int rr = (32 / SC) * i + lane / SC, row = row0 + rr;
+        const float v = stage[rr * SC + (((c >> 2) ^ ((rr >> SH) & (P - 1))) << 2) + (c & 3)];
+        if (row < p.M && n < p.N) {
+          float* dst = cbase + (int64_t)row * p.ldc + n;
+          float o = p.alpha * v;
+          if (p.beta != 0.f) o = fmaf(p.beta, *dst, o);
+          *dst = o;
+        }
+      }
     }
-    __syncwarp();  // the staging buffer is refilled by the next half
+    __syncwarp();  // the staging buffer is refilled by the next part
   }
 }
 
 template <int BN, int STAGES, bool TF32, bool GROUPED>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(TcCfg<BN, STAGES, TF32>::THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs p,
                    const GroupArgs g) {
   using Cfg = TcCfg<BN, STAGES, TF32>;
@@ -218,15 +265,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&accf_bar[a], 1);
-      mbar_init(&acce_bar[a], 128);
+      mbar_init(&acce_bar[a], 32 * Cfg::EPI_WARPS);
     }
     fence_barrier_init();
   }
-  if (!GROUPED && warp == 4 && lane == 0) {
+  if (!GROUPED && warp == Cfg::EPI_WARPS && lane == 0) {
     tma_prefetch(&tmA);
     tma_prefetch(&tmB);
   }
-  if (warp == 5) tmem_alloc<Cfg::TMEM_COLS>(&tmem_base_sh);
+  if (warp == Cfg::EPI_WARPS + 1) tmem_alloc<Cfg::TMEM_COLS>(&tmem_base_sh);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -236,7 +283,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   pdl_wait();
   pdl_launch_dependents();
 
-  if (warp == 4) {
+  if (warp == Cfg::EPI_WARPS) {
     // ---------------------------------------------------------------- TMA producer
     if (elect_one()) {
       int stage = 0;
@@ -289,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp == 5) {
+  } else if (warp == Cfg::EPI_WARPS + 1) {
     // ---------------------------------------------------------------- MMA issuer
     if (elect_one()) {
       int stage = 0;
@@ -343,23 +390,26 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else {
-    // ---------------------------------------------------------------- epilogue (warps 0..3)
+    // ---------------------------------------------------------------- epilogue (warps 0..EPI_WARPS - 1)
     int acc = 0;
     uint32_t acc_phase = 0;
     for (int tile = unit0; tile < p.num_tiles; tile += units) {
       if (!mbar_wait(&accf_bar[acc], acc_phase, p.status, kStatusTimeoutAcc)) break;
       tc_fence_after();
       const TileLoc L = locate<GROUPED>(p, g, &tmA, &tmB, tile);
-      const int row0 = L.tm * kBM + warp * 32;
+      const int quad = warp & 3, row0 = L.tm * kBM + quad * 32;
+      constexpr int COLS = BN / (Cfg::EPI_WARPS / 4);  // columns of this warp
+      const int col0 = (warp >> 2) * COLS;
       float* cbase = L.C + (int64_t)L.b * L.strideC;
-      float* stage = reinterpret_cast<float*>(smem + STAGES * Cfg::STAGE_BYTES) + warp * 32 * 16;
-      const uint32_t tbase = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * BN);
+      float* stage = reinterpret_cast<float*>(smem + STAGES * Cfg::STAGE_BYTES) + warp * 32 * Cfg::STORE_COLS;
+      const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
+      for (int c0 = col0; c0 < col0 + COLS; c0 += 32) {
         uint32_t r[32];
         tmem_ld_32x32b_x32(tbase + (uint32_t)c0, r);
         tmem_ld_wait();
-        if (row0 < L.M && L.tn * BN + c0 < L.N) store_chunk32(L, cbase, row0, L.tn * BN + c0, stage, r, lane);
+        if (row0 < L.M && L.tn * BN + c0 < L.N)
+          store_chunk32<Cfg::STORE_COLS>(L, cbase, row0, L.tn * BN + c0, stage, r, lane);
       }
       tc_fence_before();
       mbar_arrive(&acce_bar[acc]);
@@ -371,7 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   __syncthreads();
-  if (warp == 5) {
+  if (warp == Cfg::EPI_WARPS + 1) {
     tc_fence_after();
     tmem_dealloc<Cfg::TMEM_COLS>(tmem_base);
   }
