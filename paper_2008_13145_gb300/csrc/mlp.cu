@@ -24,110 +24,218 @@ constexpr int NI = 7, NH = 64, NO = 8, NP = GEMM_MLP_PARAMS;
 constexpr int OW1 = 0, OB1 = OW1 + NI * NH, OW2 = OB1 + NH, OB2 = OW2 + NH * NH, OW3 = OB2 + NH, OB3 = OW3 + NH * NO;
 static_assert(OB3 + NO == NP, "parameter layout");
 
-constexpr int kChunk = 32;     // samples per block in training
+constexpr int kChunk = 16;       // samples a training block handles at a time
+constexpr int kMaxBlocks = 256;  // training blocks; each takes as many chunks as that needs
 constexpr int kThreads = 256;
+constexpr int kT = NH + 2;       // row pitch of the transposed W2
+constexpr int kCountParts = 32;  // partial counts of the measured outputs
+
+int grad_chunks(int n) {  // chunks per block
+  const int chunks = (n + kChunk - 1) / kChunk;
+  return (chunks + kMaxBlocks - 1) / kMaxBlocks;
+}
+int grad_blocks(int n) {
+  const int per = kChunk * grad_chunks(n);
+  return (n + per - 1) / per;
+}
 
 struct GradArgs {
-  int n;
+  int n, chunks;
   const float* P;
   const float* X;
   const float* T;
   const float* mask;
-  const float* count;  // device scalar: number of measured outputs
+  const float* count;  // kCountParts partial counts of measured outputs; unused without a mask
   float* partials;     // nblocks x NP
   float* loss_part;    // nblocks
   int* step;           // Adam step counter, incremented by block 0 (may be null)
 };
 
+// Forward pass, masked squared-error gradient and partial parameter gradient of
+// a block's chunks.  Bound by shared-memory loads (about 30 MFLOP at 2,000
+// samples are nothing): a warp takes two samples and its lanes two units each,
+// so weights arrive as one 8-byte load per lane and activations as broadcasts of
+// four, and each thread accumulates a 4 x 4 tile of W2's gradient.  W2 is kept
+// transposed too: reading a column of it per lane cost a 32-way bank conflict.
+// 2,000 samples, whole call: 35 us with a one-block count, chunks of 32 on 63 SMs and
+// one output a thread; 18 us so, on 125 SMs (the host issues it in about that).
 __global__ void __launch_bounds__(kThreads) mlp_grad_kernel(const GradArgs a) {
   extern __shared__ float sm[];
   float* P = sm;                      // NP
-  float* x = P + NP;                  // kChunk x NI
-  float* z1 = x + kChunk * NI;        // kChunk x NH
-  float* z2 = z1 + kChunk * NH;       // kChunk x NH
-  float* dy = z2 + kChunk * NH;       // kChunk x NO
-  float* d2 = dy + kChunk * NO;       // kChunk x NH
+  float* W2T = P + NP;                // NH x kT: W2T[j][i] = W2[i][j]
+  float* h1 = W2T + NH * kT;          // kChunk x NH, each layer after its ReLU
+  float* h2 = h1 + kChunk * NH;       // kChunk x NH
+  float* d2 = h2 + kChunk * NH;       // kChunk x NH
   float* d1 = d2 + kChunk * NH;       // kChunk x NH
+  float* dy = d1 + kChunk * NH;       // kChunk x NO
+  float* x = dy + kChunk * NO;        // kChunk x NI
   __shared__ float red[kThreads / 32];
-  const int tid = threadIdx.x, s0 = blockIdx.x * kChunk;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (a.step && blockIdx.x == 0 && tid == 0) atomicAdd(a.step, 1);
-  for (int p = tid; p < NP; p += kThreads) P[p] = a.P[p];
-  for (int e = tid; e < kChunk * NI; e += kThreads) {
-    const int s = s0 + e / NI;
-    x[e] = s < a.n ? a.X[(int64_t)s * NI + e % NI] : 0.f;
-  }
-  __syncthreads();
-  for (int e = tid; e < kChunk * NH; e += kThreads) {
-    const int s = e / NH, j = e % NH;
-    float z = P[OB1 + j];
-    for (int i = 0; i < NI; ++i) z = fmaf(x[s * NI + i], P[OW1 + i * NH + j], z);
-    z1[e] = z;
-  }
-  __syncthreads();
-  for (int e = tid; e < kChunk * NH; e += kThreads) {
-    const int s = e / NH, j = e % NH;
-    float z = P[OB2 + j];
-    for (int i = 0; i < NH; ++i) z = fmaf(fmaxf(z1[s * NH + i], 0.f), P[OW2 + i * NH + j], z);
-    z2[e] = z;
-  }
-  __syncthreads();
-  const float inv = 1.f / *a.count;
-  float lsum = 0.f;
-  for (int e = tid; e < kChunk * NO; e += kThreads) {
-    const int s = e / NO, o = e % NO, gs = s0 + s;
-    float y = P[OB3 + o];
-    for (int i = 0; i < NH; ++i) y = fmaf(fmaxf(z2[s * NH + i], 0.f), P[OW3 + i * NO + o], y);
-    float r = 0.f;
-    if (gs < a.n) {
-      const float m = a.mask ? a.mask[(int64_t)gs * NO + o] : 1.f;
-      r = (y - a.T[(int64_t)gs * NO + o]) * m;
-    }
-    lsum = fmaf(r, r, lsum);
-    dy[e] = 2.f * r * inv;
-  }
-  __syncthreads();
-  for (int e = tid; e < kChunk * NH; e += kThreads) {
-    const int s = e / NH, i = e % NH;
-    float g = 0.f;
-    for (int o = 0; o < NO; ++o) g = fmaf(dy[s * NO + o], P[OW3 + i * NO + o], g);
-    d2[e] = z2[e] > 0.f ? g : 0.f;
-  }
-  __syncthreads();
-  for (int e = tid; e < kChunk * NH; e += kThreads) {
-    const int s = e / NH, i = e % NH;
-    float g = 0.f;
-    for (int j = 0; j < NH; ++j) g = fmaf(d2[s * NH + j], P[OW2 + i * NH + j], g);
-    d1[e] = z1[e] > 0.f ? g : 0.f;
-  }
-  __syncthreads();
-  float* out = a.partials + (int64_t)blockIdx.x * NP;
   for (int p = tid; p < NP; p += kThreads) {
-    float g = 0.f;
-    if (p < OB1) {
-      const int i = p / NH, j = p % NH;
-      for (int s = 0; s < kChunk; ++s) g = fmaf(x[s * NI + i], d1[s * NH + j], g);
-    } else if (p < OW2) {
-      const int j = p - OB1;
-      for (int s = 0; s < kChunk; ++s) g += d1[s * NH + j];
-    } else if (p < OB2) {
-      const int i = (p - OW2) / NH, j = (p - OW2) % NH;
-      for (int s = 0; s < kChunk; ++s) g = fmaf(fmaxf(z1[s * NH + i], 0.f), d2[s * NH + j], g);
-    } else if (p < OW3) {
-      const int j = p - OB2;
-      for (int s = 0; s < kChunk; ++s) g += d2[s * NH + j];
-    } else if (p < OB3) {
-      const int i = (p - OW3) / NO, o = (p - OW3) % NO;
-      for (int s = 0; s < kChunk; ++s) g = fmaf(fmaxf(z2[s * NH + i], 0.f), dy[s * NO + o], g);
-    } else {
-      const int o = p - OB3;
-      for (int s = 0; s < kChunk; ++s) g += dy[s * NO + o];
+    const float v = a.P[p];
+    P[p] = v;
+    if (p >= OW2 && p < OB2) W2T[(p - OW2) % NH * kT + (p - OW2) / NH] = v;
+  }
+  float gw2[4][4] = {}, rest[5] = {};  // this thread's gradient entries, summed over the chunks
+  float lsum = 0.f, inv = 0.f;
+  for (int c = 0; c < a.chunks; ++c) {
+    const int s0 = (blockIdx.x * a.chunks + c) * kChunk;
+    if (s0 >= a.n) break;
+    __syncthreads();  // weights stored; the last chunk's activations read
+    if (tid < kChunk * NI) x[tid] = s0 + tid / NI < a.n ? a.X[(int64_t)s0 * NI + tid] : 0.f;
+    __syncthreads();
+    const int s = 2 * warp, j = 2 * lane;  // two samples, two units
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      float2 z = *reinterpret_cast<const float2*>(P + OB1 + j);
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const float2 w = *reinterpret_cast<const float2*>(P + OW1 + i * NH + j);
+        const float xi = x[(s + u) * NI + i];
+        z.x = fmaf(xi, w.x, z.x);
+        z.y = fmaf(xi, w.y, z.y);
+      }
+      *reinterpret_cast<float2*>(h1 + (s + u) * NH + j) = make_float2(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f));
     }
-    out[p] = g;
+    __syncwarp();  // a warp reads only its own samples up to the parameter gradients
+    {
+      float2 z0 = *reinterpret_cast<const float2*>(P + OB2 + j), z1 = z0;
+#pragma unroll 4
+      for (int i = 0; i < NH; i += 4) {
+        const float4 u0 = *reinterpret_cast<const float4*>(h1 + s * NH + i);
+        const float4 u1 = *reinterpret_cast<const float4*>(h1 + (s + 1) * NH + i);
+        const float e0[4] = {u0.x, u0.y, u0.z, u0.w}, e1[4] = {u1.x, u1.y, u1.z, u1.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 w = *reinterpret_cast<const float2*>(P + OW2 + (i + q) * NH + j);
+          z0.x = fmaf(e0[q], w.x, z0.x); z0.y = fmaf(e0[q], w.y, z0.y);
+          z1.x = fmaf(e1[q], w.x, z1.x); z1.y = fmaf(e1[q], w.y, z1.y);
+        }
+      }
+      *reinterpret_cast<float2*>(h2 + s * NH + j) = make_float2(fmaxf(z0.x, 0.f), fmaxf(z0.y, 0.f));
+      *reinterpret_cast<float2*>(h2 + (s + 1) * NH + j) = make_float2(fmaxf(z1.x, 0.f), fmaxf(z1.y, 0.f));
+    }
+    __syncwarp();
+    if (c == 0) {
+      // The count comes from the kernel before, which this one may overlap up to here.
+      pdl_wait();
+      float t = (float)a.n * NO;
+      if (a.mask) {
+        t = a.count[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      }
+      inv = 1.f / (t > 0.f ? t : 1.f);
+    }
+    {  // outputs: 16 of the warp's two samples, two lanes (halves of the sum) each
+      const int ss = s + (lane >> 4), o = (lane >> 1) & 7, k0 = (lane & 1) * (NH / 2), gs = s0 + ss;
+      float y = (lane & 1) ? 0.f : P[OB3 + o];
+#pragma unroll 8
+      for (int i = k0; i < k0 + NH / 2; ++i) y = fmaf(h2[ss * NH + i], P[OW3 + i * NO + o], y);
+      y += __shfl_xor_sync(0xffffffffu, y, 1);
+      if (!(lane & 1)) {
+        float r = 0.f;
+        if (gs < a.n) {
+          const float m = a.mask ? a.mask[(int64_t)gs * NO + o] : 1.f;
+          r = (y - a.T[(int64_t)gs * NO + o]) * m;
+        }
+        lsum = fmaf(r, r, lsum);
+        dy[ss * NO + o] = 2.f * r * inv;
+      }
+    }
+    __syncwarp();
+    {
+      float w[2][NO];
+#pragma unroll
+      for (int v = 0; v < 2; ++v)
+#pragma unroll
+        for (int o = 0; o < NO; o += 4) {
+          const float4 t = *reinterpret_cast<const float4*>(P + OW3 + (j + v) * NO + o);
+          w[v][o] = t.x; w[v][o + 1] = t.y; w[v][o + 2] = t.z; w[v][o + 3] = t.w;
+        }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float2 g = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int o = 0; o < NO; ++o) {
+          const float d = dy[(s + u) * NO + o];
+          g.x = fmaf(d, w[0][o], g.x);
+          g.y = fmaf(d, w[1][o], g.y);
+        }
+        const float2 h = *reinterpret_cast<const float2*>(h2 + (s + u) * NH + j);
+        *reinterpret_cast<float2*>(d2 + (s + u) * NH + j) = make_float2(h.x > 0.f ? g.x : 0.f, h.y > 0.f ? g.y : 0.f);
+      }
+    }
+    __syncwarp();
+    {
+      float2 g0 = make_float2(0.f, 0.f), g1 = g0;
+#pragma unroll 4
+      for (int q0 = 0; q0 < NH; q0 += 4) {
+        const float4 u0 = *reinterpret_cast<const float4*>(d2 + s * NH + q0);
+        const float4 u1 = *reinterpret_cast<const float4*>(d2 + (s + 1) * NH + q0);
+        const float e0[4] = {u0.x, u0.y, u0.z, u0.w}, e1[4] = {u1.x, u1.y, u1.z, u1.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 w = *reinterpret_cast<const float2*>(W2T + (q0 + q) * kT + j);
+          g0.x = fmaf(e0[q], w.x, g0.x); g0.y = fmaf(e0[q], w.y, g0.y);
+          g1.x = fmaf(e1[q], w.x, g1.x); g1.y = fmaf(e1[q], w.y, g1.y);
+        }
+      }
+      const float2 a0 = *reinterpret_cast<const float2*>(h1 + s * NH + j);
+      const float2 a1 = *reinterpret_cast<const float2*>(h1 + (s + 1) * NH + j);
+      *reinterpret_cast<float2*>(d1 + s * NH + j) = make_float2(a0.x > 0.f ? g0.x : 0.f, a0.y > 0.f ? g0.y : 0.f);
+      *reinterpret_cast<float2*>(d1 + (s + 1) * NH + j) = make_float2(a1.x > 0.f ? g1.x : 0.f, a1.y > 0.f ? g1.y : 0.f);
+    }
+    __syncthreads();
+    {
+      const int i4 = 4 * (tid >> 4), j4 = 4 * (tid & 15);
+#pragma unroll 4
+      for (int t = 0; t < kChunk; ++t) {
+        const float4 u = *reinterpret_cast<const float4*>(h1 + t * NH + i4);
+        const float4 v = *reinterpret_cast<const float4*>(d2 + t * NH + j4);
+        const float uu[4] = {u.x, u.y, u.z, u.w}, vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int w = 0; w < 4; ++w) gw2[q][w] = fmaf(uu[q], vv[w], gw2[q][w]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {  // W1, b1, b2, W3, b3 in turn
+      int p = tid + k * kThreads;
+      if (p >= OW2) p += NH * NH;
+      if (p >= NP) continue;
+      float g = rest[k];
+      if (p < OB1) {
+        for (int t = 0; t < kChunk; ++t) g = fmaf(x[t * NI + p / NH], d1[t * NH + p % NH], g);
+      } else if (p < OW2) {
+        for (int t = 0; t < kChunk; ++t) g += d1[t * NH + p - OB1];
+      } else if (p < OW3) {
+        for (int t = 0; t < kChunk; ++t) g += d2[t * NH + p - OB2];
+      } else if (p < OB3) {
+        for (int t = 0; t < kChunk; ++t) g = fmaf(h2[t * NH + (p - OW3) / NO], dy[t * NO + (p - OW3) % NO], g);
+      } else {
+        for (int t = 0; t < kChunk; ++t) g += dy[t * NO + p - OB3];
+      }
+      rest[k] = g;
+    }
+  }
+  float* out = a.partials + (int64_t)blockIdx.x * NP;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    *reinterpret_cast<float4*>(out + OW2 + (4 * (tid >> 4) + q) * NH + 4 * (tid & 15)) =
+        make_float4(gw2[q][0], gw2[q][1], gw2[q][2], gw2[q][3]);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    int p = tid + k * kThreads;
+    if (p >= OW2) p += NH * NH;
+    if (p < NP) out[p] = rest[k];
   }
   // block loss partial (sum of squared masked residuals / count)
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-  if ((tid & 31) == 0) red[tid >> 5] = lsum;
+  if (lane == 0) red[warp] = lsum;
   __syncthreads();
   if (tid == 0) {
     float t = 0.f;
@@ -136,34 +244,58 @@ __global__ void __launch_bounds__(kThreads) mlp_grad_kernel(const GradArgs a) {
   }
 }
 
-__global__ void mlp_reduce_kernel(const float* partials, const float* loss_part, int nblocks, float* grad,
-                                  float* loss, float* loss_hist, const int* step, int t0) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+// Sums the blocks' partials in a fixed order: 32 parameters a block, each by
+// eight threads that take every eighth block's.  (One thread per parameter
+// walked 63 partials in 8 us.)  Block 0 also sums the loss.
+__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float* partials, const float* loss_part, int nblocks,
+                                                         float* grad, float* loss, float* loss_hist, const int* step,
+                                                         int t0) {
+  __shared__ float part[8][33];
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31, p = blockIdx.x * 32 + lane;
+  pdl_wait();
+  float g = 0.f;
   if (p < NP) {
-    float g = 0.f;
-    for (int b = 0; b < nblocks; ++b) g += partials[(int64_t)b * NP + p];
-    grad[p] = g;
+#pragma unroll 8
+    for (int b = q; b < nblocks; b += 8) g += partials[(int64_t)b * NP + p];
   }
-  if (p == 0) {
+  part[q][lane] = g;
+  __syncthreads();
+  if (q == 0) {
+    if (p < NP) {
+      float t = part[0][lane];
+#pragma unroll
+      for (int u = 1; u < 8; ++u) t += part[u][lane];
+      grad[p] = t;
+    }
+  } else if (q == 1 && blockIdx.x == 0) {
     float l = 0.f;
-    for (int b = 0; b < nblocks; ++b) l += loss_part[b];
-    if (loss) *loss = l;
-    if (loss_hist && step) loss_hist[*step - t0 - 1] = l;
+    for (int b = lane; b < nblocks; b += 32) l += loss_part[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) {
+      if (loss) *loss = l;
+      if (loss_hist && step) loss_hist[*step - t0 - 1] = l;
+    }
   }
 }
 
-__global__ void mlp_count_kernel(const float* mask, int64_t total, float* count) {
-  __shared__ float red[32];
+// Partial sums of the mask, one per block of the kCountParts that the gradient kernel adds.
+__global__ void __launch_bounds__(256) mlp_count_kernel(const float* mask, int64_t total, float* count) {
+  __shared__ float red[8];
+  pdl_launch_dependents();  // the gradient kernel's forward pass reads nothing that is written here
   float c = 0.f;
-  for (int64_t i = threadIdx.x; i < total; i += blockDim.x) c += mask ? mask[i] : 1.f;
+  const int64_t each = (total + kCountParts - 1) / kCountParts, first = blockIdx.x * each;
+  const int64_t last = first + each < total ? first + each : total;
+#pragma unroll 4
+  for (int64_t i = first + threadIdx.x; i < last; i += blockDim.x) c += mask[i];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
   __syncthreads();
   if (threadIdx.x == 0) {
     float t = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    *count = t > 0.f ? t : 1.f;
+    for (int w = 0; w < 8; ++w) t += red[w];
+    count[blockIdx.x] = t;
   }
 }
 
@@ -270,7 +402,7 @@ gemm_status_t fail(cudaError_t e) {
   return GEMM_ERR_CUDA;
 }
 
-constexpr size_t kGradSmem = sizeof(float) * (NP + kChunk * NI + 4 * kChunk * NH + kChunk * NO);
+constexpr size_t kGradSmem = sizeof(float) * (NP + NH * kT + kChunk * (4 * NH + NO + NI));
 
 cudaError_t ensure_attr() {
   static unsigned long long done = 0;
@@ -295,7 +427,7 @@ struct Workspace {
 };
 
 cudaError_t ws_alloc(int nblocks, cudaStream_t s, Workspace* w) {
-  const size_t bytes = sizeof(float) * ((size_t)nblocks * NP + nblocks + 1 + NP + 1) + sizeof(int) + 6 * 256;
+  const size_t bytes = sizeof(float) * ((size_t)nblocks * NP + nblocks + kCountParts + NP + 1) + sizeof(int) + 6 * 256;
   cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&w->base), bytes, s);
   if (e != cudaSuccess) return e;
   char* p = w->base;
@@ -306,7 +438,7 @@ cudaError_t ws_alloc(int nblocks, cudaStream_t s, Workspace* w) {
   };
   w->partials = reinterpret_cast<float*>(carve(sizeof(float) * (size_t)nblocks * NP));
   w->loss_part = reinterpret_cast<float*>(carve(sizeof(float) * nblocks));
-  w->count = reinterpret_cast<float*>(carve(sizeof(float)));
+  w->count = reinterpret_cast<float*>(carve(sizeof(float) * kCountParts));
   w->grad = reinterpret_cast<float*>(carve(sizeof(float) * NP));
   w->loss = reinterpret_cast<float*>(carve(sizeof(float)));
   w->step = reinterpret_cast<int*>(carve(sizeof(int)));
@@ -315,11 +447,12 @@ cudaError_t ws_alloc(int nblocks, cudaStream_t s, Workspace* w) {
 
 // ---------------------------------------------------------------- allocation-free loss/gradient
 // Scratch of mlp_loss_grad_noalloc: per-block gradient partials for up to
-// kNoAllocMaxSamples samples, then the per-block losses, then the count of
+// kNoAllocMaxSamples samples, then the per-block losses, then the counts of
 // measured outputs.  Every device that loads the library holds this array
 // (about 5.3 MB) until the process exits.
 constexpr int kNoAllocMaxSamples = 8192;
-constexpr int kNoAllocMaxBlocks = kNoAllocMaxSamples / kChunk;
+constexpr int kNoAllocMaxBlocks = kMaxBlocks;
+static_assert(kCountParts <= 64, "the scratch holds 64 floats after the losses");
 constexpr size_t kNoAllocFloats = (size_t)kNoAllocMaxBlocks * NP + kNoAllocMaxBlocks + 64;
 static __device__ __align__(256) float g_noalloc_scratch[kNoAllocFloats];
 
@@ -344,6 +477,31 @@ float* noalloc_scratch(cudaError_t* err) {
     addr[dev] = static_cast<float*>(p);
   }
   return addr[dev];
+}
+
+// The gradient kernels of one pass: the count of measured outputs (without a mask
+// it is known), the blocks' partials, their sums.  Each may start while the one
+// before it drains; all writes and all reads of what those write come after
+// the wait.
+cudaError_t launch_count(const float* mask, int n, float* count, cudaStream_t s) {
+  if (!mask) return cudaSuccess;
+  mlp_count_kernel<<<kCountParts, 256, 0, s>>>(mask, (int64_t)n * NO, count);
+  return cudaGetLastError();
+}
+cudaError_t launch_grad(const GradArgs& a, float* grad, float* loss, float* loss_hist, int t0, bool overlap,
+                        cudaStream_t s) {
+  const int nb = grad_blocks(a.n);
+  cudaError_t e = cudaSuccess;
+  if (overlap) {
+    e = launch_pdl(mlp_grad_kernel, dim3(nb), dim3(kThreads), kGradSmem, s, nullptr, 0, a);
+  } else {
+    mlp_grad_kernel<<<nb, kThreads, kGradSmem, s>>>(a);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return e;
+  return launch_pdl(mlp_reduce_kernel, dim3((NP + 31) / 32), dim3(256), 0, s, nullptr, 0,
+                    static_cast<const float*>(a.partials), static_cast<const float*>(a.loss_part), nb, grad, loss,
+                    loss_hist, static_cast<const int*>(a.step), t0);
 }
 
 }  // namespace mlp
@@ -385,14 +543,11 @@ gemm_status_t mlp_loss_grad(int32_t n, const float* P, const float* X, const flo
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = ensure_attr();
   if (e != cudaSuccess) return fail(e);
-  const int nb = (n + kChunk - 1) / kChunk;
   Workspace w;
-  if ((e = ws_alloc(nb, s, &w)) != cudaSuccess) return fail(e);
-  mlp_count_kernel<<<1, 256, 0, s>>>(mask, (int64_t)n * NO, w.count);
-  GradArgs a{n, P, X, T, mask, w.count, w.partials, w.loss_part, nullptr};
-  mlp_grad_kernel<<<nb, kThreads, kGradSmem, s>>>(a);
-  mlp_reduce_kernel<<<(NP + 255) / 256, 256, 0, s>>>(w.partials, w.loss_part, nb, grad, loss, nullptr, nullptr, 0);
-  e = cudaGetLastError();
+  if ((e = ws_alloc(grad_blocks(n), s, &w)) != cudaSuccess) return fail(e);
+  GradArgs a{n, grad_chunks(n), P, X, T, mask, w.count, w.partials, w.loss_part, nullptr};
+  e = launch_count(mask, n, w.count, s);
+  if (e == cudaSuccess) e = launch_grad(a, grad, loss, nullptr, 0, mask != nullptr, s);
   cudaFreeAsync(w.base, s);
   return e == cudaSuccess ? GEMM_OK : fail(e);
 }
@@ -409,14 +564,11 @@ gemm_status_t mlp_loss_grad_noalloc(int32_t n, const float* P, const float* X, c
   float* partials = base;
   float* loss_part = base + (size_t)kNoAllocMaxBlocks * NP;
   float* count = loss_part + kNoAllocMaxBlocks;
-  // Every scratch value read below is written earlier in this call (count, then
-  // the partials and losses of blocks 0..nb-1), so nothing needs clearing.
-  const int nb = (n + kChunk - 1) / kChunk;
-  mlp_count_kernel<<<1, 256, 0, s>>>(mask, (int64_t)n * NO, count);
-  GradArgs a{n, P, X, T, mask, count, partials, loss_part, nullptr};
-  mlp_grad_kernel<<<nb, kThreads, kGradSmem, s>>>(a);
-  mlp_reduce_kernel<<<(NP + 255) / 256, 256, 0, s>>>(partials, loss_part, nb, grad, loss, nullptr, nullptr, 0);
-  e = cudaGetLastError();
+  // Every scratch value read below is written earlier in this call (the counts,
+  // then the partials and losses of the blocks), so nothing needs clearing.
+  GradArgs a{n, grad_chunks(n), P, X, T, mask, count, partials, loss_part, nullptr};
+  e = launch_count(mask, n, count, s);
+  if (e == cudaSuccess) e = launch_grad(a, grad, loss, nullptr, 0, mask != nullptr, s);
   return e == cudaSuccess ? GEMM_OK : fail(e);
 }
 
@@ -437,11 +589,10 @@ gemm_status_t mlp_train(int32_t n, float* P, const float* X, const float* T, con
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = ensure_attr();
   if (e != cudaSuccess) return fail(e);
-  const int nb = (n + kChunk - 1) / kChunk;
   Workspace w;
-  if ((e = ws_alloc(nb, s, &w)) != cudaSuccess) return fail(e);
-  mlp_count_kernel<<<1, 256, 0, s>>>(mask, (int64_t)n * NO, w.count);
-  e = cudaMemcpyAsync(w.step, &t0, sizeof(int), cudaMemcpyHostToDevice, s);
+  if ((e = ws_alloc(grad_blocks(n), s, &w)) != cudaSuccess) return fail(e);
+  e = launch_count(mask, n, w.count, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(w.step, &t0, sizeof(int), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaStream_t cap = nullptr;
   cudaGraph_t graph = nullptr;
@@ -449,13 +600,11 @@ gemm_status_t mlp_train(int32_t n, float* P, const float* X, const float* T, con
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    GradArgs a{n, P, X, T, mask, w.count, w.partials, w.loss_part, w.step};
-    mlp_grad_kernel<<<nb, kThreads, kGradSmem, cap>>>(a);
-    mlp_reduce_kernel<<<(NP + 255) / 256, 256, 0, cap>>>(w.partials, w.loss_part, nb, w.grad, w.loss, loss_hist,
-                                                         w.step, t0);
+    GradArgs a{n, grad_chunks(n), P, X, T, mask, w.count, w.partials, w.loss_part, w.step};
+    cudaError_t el = launch_grad(a, w.grad, w.loss, loss_hist, t0, false, cap);
     mlp_adam_kernel<<<(NP + 255) / 256, 256, 0, cap>>>(P, w.grad, m, v, w.step, 0, lr, b1, b2, eps);
     cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
-    e = (e2 != cudaSuccess) ? e2 : cudaGetLastError();
+    e = (e2 != cudaSuccess) ? e2 : el != cudaSuccess ? el : cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
   for (int i = 0; i < steps && e == cudaSuccess; ++i) e = cudaGraphLaunch(exec, s);
