@@ -753,11 +753,14 @@ struct UploadChunk {
   alignas(16) uint8_t data[kUploadBytes];
 };
 
-__global__ void upload_kernel(const __grid_constant__ UploadChunk c) {
-  const int n16 = c.n / 16;
-  for (int i = threadIdx.x; i < n16; i += blockDim.x)
-    reinterpret_cast<uint4*>(c.dst)[i] = reinterpret_cast<const uint4*>(c.data)[i];
-  for (int i = n16 * 16 + threadIdx.x; i < c.n; i += blockDim.x) c.dst[i] = c.data[i];
+// 16 bytes a thread over as many small blocks as that takes: parameters are read
+// through the constant cache, one address at a time, so a single block took 10 us
+// for a chunk.
+constexpr int kUploadThreads = 32;
+__global__ void __launch_bounds__(kUploadThreads) upload_kernel(const __grid_constant__ UploadChunk c) {
+  const int n16 = c.n / 16, i = blockIdx.x * kUploadThreads + threadIdx.x;
+  if (i < n16) reinterpret_cast<uint4*>(c.dst)[i] = reinterpret_cast<const uint4*>(c.data)[i];
+  if (blockIdx.x == 0 && n16 * 16 + threadIdx.x < c.n) c.dst[n16 * 16 + threadIdx.x] = c.data[n16 * 16 + threadIdx.x];
 }
 
 cudaError_t upload(void* dst, const void* src, size_t bytes, cudaStream_t s) {
@@ -767,7 +770,7 @@ cudaError_t upload(void* dst, const void* src, size_t bytes, cudaStream_t s) {
     ch->dst = static_cast<uint8_t*>(dst) + off;
     ch->n = (int)std::min<size_t>(kUploadBytes, bytes - off);
     std::memcpy(ch->data, static_cast<const uint8_t*>(src) + off, ch->n);
-    upload_kernel<<<1, 256, 0, s>>>(*ch);
+    upload_kernel<<<ch->n / 16 / kUploadThreads + 1, kUploadThreads, 0, s>>>(*ch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
