@@ -86,7 +86,9 @@ gemm_status_t kselect_debug_shrink_extents(int64_t a_bytes, int64_t b_bytes, int
  * 0..575.  Tensor-core families (ids 1000 + 100*(family-1) + index, index =
  * (BN slot * 3 + stage slot) * 2) use a 128 x BN tile per CTA with BN in
  * {64,128,256} and a shared-memory ring of {2,3,4} stages: 9 configs per family
- * (the odd indexes are reserved and name no kernel: GEMM_ERR_NO_KERNEL).
+ * (the odd indexes are reserved and name no kernel: GEMM_ERR_NO_KERNEL).  The
+ * launcher runs BN 256 on pairs of CTAs that share a 256 x 256 tile where that
+ * is expected to be faster (the same results; not in grouped launches).
  * gemm_config_id(family, i) = 1000 + 100*(family-1) + 2*i.  Operands are read in place by
  * TMA when K- or MN-contiguous (TF32 and BF16), 16-byte aligned and
  * batch-packed; others, and every F32X3 operand (split once into BF16 hi and

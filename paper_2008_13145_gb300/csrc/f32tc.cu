@@ -628,42 +628,6 @@ struct Pair {
   static constexpr int TMEM = 512;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// The address of a shared-memory word of ours in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-// What an arrival announces (operand parts, emptied accumulators) is read by
-// the announcing SM's own tensor core and is ordered by the proxy and tcgen05
-// fences before it, so it needs no cluster-wide release (which would wait over
-// 1000 clocks for every write under way).
-__device__ __forceinline__ void arrive_cluster(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accum));
-}
-// Arrives on the barrier at this offset in both CTAs once the MMAs issued so far are complete.
-__device__ __forceinline__ void commit_pair(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_u32(bar)),
-      "h"((uint16_t)3)
-      : "memory");
-}
-
 // A converting group of the pair kernel: its operand's 128 rows of every chunk.
 template <class S>
 __device__ __forceinline__ void convert_pair(const Args& p, int total, bool is_a, uint32_t rank, uint32_t smem,
@@ -760,11 +724,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     fence_barrier_init();
   }
   if (threadIdx.x < kMarks) inexact[threadIdx.x] = 0;
-  if (warp == kIssuer) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sh)),
-                 "r"(Pair::TMEM));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
-  }
+  if (warp == kIssuer) tmem_alloc_pair<Pair::TMEM>(&tmem_sh);
   tc_fence_before();
   __syncthreads();
   cluster_sync();
@@ -791,7 +751,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         for (int g = 0; g < 6; ++g)
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            mma_pair(d, da + (pa[g] * Pair::PART + k * 32) / 16, db + (pb[g] * Pair::PART + k * 32) / 16, idesc,
+            mma_pair<false>(d, da + (pa[g] * Pair::PART + k * 32) / 16, db + (pb[g] * Pair::PART + k * 32) / 16, idesc,
                      (g | k) != 0 ? 1u : 0u);
         commit_pair(&empty[stage]);
         commit_pair(&accf[i & 1]);
@@ -853,7 +813,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync();  // neither CTA leaves while the other's MMAs or arrivals may reach it
   if (warp == kIssuer) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Pair::TMEM));
+    tmem_dealloc_pair<Pair::TMEM>(tmem);
   }
 }
 

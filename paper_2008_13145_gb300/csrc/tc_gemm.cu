@@ -403,6 +403,38 @@ cudaError_t launch_kernel(const CUtensorMap& ma, const CUtensorMap& mb, const tc
                     nullptr, 0, ma, mb, a, g);
 }
 
+// The 256 x 256 tiles of CTA pairs, one pair per two SMs.
+template <bool TF32>
+cudaError_t launch_pair(const CUtensorMap& ma, const CUtensorMap& mb, const tc::TcArgs& a, int sms, cudaStream_t s) {
+  using Cfg = tc::PairCfg<TF32>;
+  auto kern = tc::tc_pair_kernel<TF32>;
+  static unsigned long long done_mask = 0;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (!(__atomic_load_n(&done_mask, __ATOMIC_ACQUIRE) & bit)) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    __atomic_fetch_or(&done_mask, bit, __ATOMIC_ACQ_REL);
+  }
+  const int pairs = std::min(a.num_tiles, sms / 2);
+  return launch_pdl(kern, dim3((unsigned)(2 * pairs)), dim3(Cfg::THREADS), (size_t)Cfg::SMEM_BYTES, s, nullptr, 0, ma,
+                    mb, a);
+}
+
+// Whether a BN 256 request runs on CTA pairs: where their rounds of tiles, at
+// 0.85 of a single CTA's time for the same products (0.79 to 0.84 measured where
+// both have the same rounds, 8192 and 4096 cubed; 0.85 with 12 rounds to 11 at
+// 3634 x 1714 x 406 x 8), come out no longer.  One row of tiles stays single: the
+// second CTA would have none.  The `stages` of the config do not apply to pairs.
+bool use_pair(const TcConfig& c, const GemmArgs& g, int sms) {
+  if (c.bn != 256 || sms < 2 || g.M <= 128) return false;
+  const int64_t cols = ((int64_t)g.N + 255) / 256 * g.batch;
+  const int64_t singles = ((int64_t)g.M + 127) / 128 * cols, pairs = ((int64_t)g.M + 255) / 256 * cols;
+  const int64_t rounds1 = (singles + sms - 1) / sms, rounds2 = (pairs + sms / 2 - 1) / (sms / 2);
+  return 0.85 * rounds2 <= rounds1;
+}
+
 using TcLaunch = cudaError_t (*)(const CUtensorMap&, const CUtensorMap&, const tc::TcArgs&, const tc::GroupArgs&,
                                  cudaStream_t);
 
@@ -517,7 +549,11 @@ gemm_status_t tc_launch(int id, const GemmArgs& g, cudaStream_t s) {
   if (!status) return fail(cudaGetLastError());
 
   // op(A) rows are M, stored M x K when transA = 0; op(B)^T rows are N, stored N x K when transB = 1.
-  const int b_ext = c.bn;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return fail(cudaGetLastError());
+  const bool pair = use_pair(c, g, sms);
+  const int b_ext = pair ? 128 : c.bn;  // rows of B^T that one CTA loads per slice
   OperandPlan pa = plan_operand(c, g.A, g.lda, g.strideA, !g.transA, g.M, g.K, g.batch, tc::kBM);
   OperandPlan pb = plan_operand(c, g.B, g.ldb, g.strideB, g.transB != 0, g.N, g.K, g.batch, b_ext);
   char* scratch = nullptr;
@@ -555,14 +591,14 @@ gemm_status_t tc_launch(int id, const GemmArgs& g, cudaStream_t s) {
   if (st == GEMM_OK) {
     tc::TcArgs a;
     a.M = g.M; a.N = g.N; a.K = (int)Kop; a.batch = g.batch;
-    a.tiles_m = row_tiles(g.M);
+    a.tiles_m = pair ? (g.M + 255) / 256 : row_tiles(g.M);
     a.tiles_n = (g.N + c.bn - 1) / c.bn;
     a.num_tiles = a.tiles_m * a.tiles_n * g.batch;
     a.k_blocks = (int)((Kop + (op_bf16 ? 63 : 31)) / (op_bf16 ? 64 : 32));
     // Grouped raster: 8 tile rows per group bound the operand slices the
     // SMs' tiles in flight read at once (8 A + ~10 B slices for 152 CTAs).
     a.raster = 2;
-    a.group_m = std::max(1, std::min(a.tiles_m, kRasterGroup));
+    a.group_m = std::max(1, std::min(a.tiles_m, pair ? kRasterGroup / 2 : kRasterGroup));
     a.alpha = g.alpha; a.beta = g.beta;
     a.C = g.C; a.ldc = g.ldc; a.strideC = g.strideC; a.vecC = vec_of(g.C, g.ldc, g.batch == 1 ? 0 : g.strideC);
     a.a_mn = pa.mn; a.b_mn = pb.mn;
@@ -570,7 +606,7 @@ gemm_status_t tc_launch(int id, const GemmArgs& g, cudaStream_t s) {
     a.seg_map = x3 ? sp.seg_map : 0;
     a.status = status;
     tc::GroupArgs none{nullptr, 0};
-    e = fn(ma, mb, a, none, s);
+    e = !pair ? fn(ma, mb, a, none, s) : op_bf16 ? launch_pair<false>(ma, mb, a, sms, s) : launch_pair<true>(ma, mb, a, sms, s);
     if (e != cudaSuccess) st = fail(e);
   }
   if (scratch) cudaFreeAsync(scratch, s);

@@ -162,10 +162,14 @@ __device__ __forceinline__ TileLoc locate(const TcArgs& p, const GroupArgs& g, c
 // epilogue warp per quadrant this took f32mix 1733 x 912 x 1408 x 2 from 77 to 48
 // us, an uneven BF16 group of 256 from 509 to 443 and, with rows of 637 floats,
 // BF16 2185 x 637 x 95 x 16 from 87 to 63 (its lanes wrote 4 bytes every 16).
-template <int SC>
+// RUNS: rows on 32 bytes go through the staging buffer too unless C is read
+// (the CTA-pair tiles: 128-byte runs took BF16 3634 x 1712 x 408 x 8 from 68 to 58
+// us; with beta != 0, f32mix 1733 x 912 x 1408 x 2, they took 54 us against 45, and
+// an uneven group of 128-row tiles 446 against 428).
+template <int SC, bool RUNS = false>
 __device__ __forceinline__ void store_chunk32(const TileLoc& p, float* cbase, int row0, int n0, float* stage,
                                               const uint32_t (&r)[32], int lane) {
-  if (p.vecC == 2 && n0 + 32 <= p.N) {
+  if (p.vecC == 2 && n0 + 32 <= p.N && !(RUNS && p.beta == 0.f)) {
     if (row0 + lane >= p.M) return;
     float* dst = cbase + (int64_t)(row0 + lane) * p.ldc + n0;
 #pragma unroll
@@ -424,6 +428,202 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, TF32>::THREADS, 1)
   if (warp == Cfg::EPI_WARPS + 1) {
     tc_fence_after();
     tmem_dealloc<Cfg::TMEM_COLS>(tmem_base);
+  }
+}
+
+// ---------------------------------------------------------------- two CTAs on one 256 x 256 tile
+// The same with tcgen05's cta_group::2: each CTA of the pair loads its 128 rows
+// of A and its 128 of B and holds its 128 rows' accumulators; the first CTA
+// issues MMAs that read both CTAs' shared memory.  A slice of K then costs an SM
+// 32 KB of loads and shared memory instead of 48 for the same products, which
+// leaves room for six stages.  What bounds the 128 x 256 tiles is feeding the
+// MMAs (36 % tensor-pipe time at 3634 x 1714 x 406 x 8 TF32).  BF16 8192 cubed A B^T
+// 685 -> 575 us (1,910 TFLOP/s), A B 672 -> 535; 4096 cubed 100 -> 80; TF32 8192
+// cubed 1360 -> 1060; TF32 3634 x 1714 x 406 x 8 102 -> 86.  Same bits.
+template <bool TF32>
+struct PairCfg {
+  static constexpr int ELEM = TF32 ? 4 : 2;
+  static constexpr int BM = 256, BN = 256, HALF = 128;
+  static constexpr int BK = 128 / ELEM, KMMA = TF32 ? 8 : 16;
+  static constexpr int PART = HALF * 128;  // bytes of one operand's half slice
+  static constexpr int STAGE_BYTES = 2 * PART, STAGES = 6;
+  static constexpr int EPI_WARPS = 8, THREADS = 32 * (EPI_WARPS + 2);
+  static constexpr int STORE_COLS = 32, EPI_BYTES = EPI_WARPS * 32 * STORE_COLS * 4;
+  static constexpr int TMEM_COLS = 2 * BN;
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024;
+  static constexpr int MN_BOX = 128 / ELEM, MN_BOX_BYTES = BK * 128;
+  static constexpr uint32_t MN_SBO = TF32 ? 512 : 1024;
+  static constexpr uint32_t MN_MODE = TF32 ? kSw128Atom32 : kSw128;
+};
+
+template <bool TF32>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<TF32>::THREADS, 1)
+    tc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs p) {
+  using Cfg = PairCfg<TF32>;
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ uint64_t full_bar[Cfg::STAGES], empty_bar[Cfg::STAGES], accf_bar[2], acce_bar[2];
+  __shared__ uint32_t tmem_base_sh;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)cluster_rank();
+  const int unit0 = (int)blockIdx.x >> 1, units = (int)gridDim.x >> 1;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < Cfg::STAGES; ++s) {
+      mbar_init(&full_bar[s], 1);  // used in the first CTA, for both CTAs' loads
+      mbar_init(&empty_bar[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&accf_bar[a], 1);
+      mbar_init(&acce_bar[a], 2 * Cfg::EPI_WARPS);  // used in the first CTA
+    }
+    fence_barrier_init();
+  }
+  if (warp == Cfg::EPI_WARPS && lane == 0) {
+    tma_prefetch(&tmA);
+    tma_prefetch(&tmB);
+  }
+  if (warp == Cfg::EPI_WARPS + 1) tmem_alloc_pair<Cfg::TMEM_COLS>(&tmem_base_sh);
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_sh;
+  pdl_wait();
+  pdl_launch_dependents();
+
+  if (warp == Cfg::EPI_WARPS) {
+    if (elect_one()) {
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int tile = unit0; tile < p.num_tiles && ok; tile += units) {
+        int b, tm, tn;
+        tile_coords(p, tile, b, tm, tn);
+        const int row = tm * Cfg::BM + rank * Cfg::HALF, col = tn * Cfg::BN + rank * Cfg::HALF;
+        for (int kb = 0; kb < p.k_blocks; ++kb) {
+          // Freed in both CTAs at once; the first CTA's full barrier is then in this
+          // slice's phase, so the other's bytes may be counted before they are expected.
+          if (!(ok = mbar_wait(&empty_bar[stage], phase ^ 1, p.status, kStatusTimeoutEmpty))) break;
+          uint8_t* sa = smem + stage * Cfg::STAGE_BYTES;
+          uint8_t* sb = sa + Cfg::PART;
+          int xa = kb * Cfg::BK, xb = kb * Cfg::BK;
+          if (!TF32 && p.seg_blocks > 0) {
+            const int g = kb / p.seg_blocks, kk = kb - g * p.seg_blocks;
+            xa = (((p.seg_map >> (2 * g)) & 3) * p.seg_blocks + kk) * Cfg::BK;
+            xb = (((p.seg_map >> (16 + 2 * g)) & 3) * p.seg_blocks + kk) * Cfg::BK;
+          }
+          const uint32_t bar = in_cta(smem_u32(&full_bar[stage]), 0);
+          if (rank == 0) mbar_arrive_expect_tx(&full_bar[stage], 2 * Cfg::STAGE_BYTES);
+          if (p.a_mn) {
+#pragma unroll
+            for (int j = 0; j < Cfg::HALF / Cfg::MN_BOX; ++j)
+              tma_load_3d_pair(sa + j * Cfg::MN_BOX_BYTES, &tmA, bar, row + j * Cfg::MN_BOX, xa, b);
+          } else {
+            tma_load_3d_pair(sa, &tmA, bar, xa, row, b);
+          }
+          if (p.b_mn) {
+#pragma unroll
+            for (int j = 0; j < Cfg::HALF / Cfg::MN_BOX; ++j)
+              tma_load_3d_pair(sb + j * Cfg::MN_BOX_BYTES, &tmB, bar, col + j * Cfg::MN_BOX, xb, b);
+          } else {
+            tma_load_3d_pair(sb, &tmB, bar, xb, col, b);
+          }
+          if (++stage == Cfg::STAGES) {
+            stage = 0;
+            phase ^= 1;
+          }
+        }
+      }
+      // Wait (bounded) until every issued slice has been read before the CTA can exit.
+      if (ok) {
+        for (int s = 0; s < Cfg::STAGES; ++s) {
+          if (!mbar_wait(&empty_bar[stage], phase ^ 1, p.status, kStatusTimeoutEmpty)) break;
+          if (++stage == Cfg::STAGES) {
+            stage = 0;
+            phase ^= 1;
+          }
+        }
+      }
+    }
+  } else if (warp == Cfg::EPI_WARPS + 1) {
+    if (rank == 0 && elect_one()) {
+      const uint32_t idesc = instr_desc<TF32>(Cfg::BM, Cfg::BN, p.a_mn != 0, p.b_mn != 0);
+      const uint32_t a_step = p.a_mn ? Cfg::KMMA * 128 : Cfg::KMMA * Cfg::ELEM;
+      const uint32_t b_step = p.b_mn ? Cfg::KMMA * 128 : Cfg::KMMA * Cfg::ELEM;
+      const uint32_t a_lbo = p.a_mn ? Cfg::MN_BOX_BYTES : 16, b_lbo = p.b_mn ? Cfg::MN_BOX_BYTES : 16;
+      const uint32_t a_sbo = p.a_mn ? Cfg::MN_SBO : 1024, b_sbo = p.b_mn ? Cfg::MN_SBO : 1024;
+      const uint32_t a_mode = p.a_mn ? Cfg::MN_MODE : kSw128, b_mode = p.b_mn ? Cfg::MN_MODE : kSw128;
+      int stage = 0, acc = 0;
+      uint32_t phase = 0, acc_phase = 0;
+      bool ok = true;
+      for (int tile = unit0; tile < p.num_tiles && ok; tile += units) {
+        if (!(ok = mbar_wait(&acce_bar[acc], acc_phase ^ 1, p.status, kStatusTimeoutAccEmpty))) break;
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * Cfg::BN);
+        for (int kb = 0; kb < p.k_blocks; ++kb) {
+          if (!(ok = mbar_wait(&full_bar[stage], phase, p.status, kStatusTimeoutFull))) break;
+          tc_fence_after();
+          const uint32_t a_addr = smem_u32(smem + stage * Cfg::STAGE_BYTES), b_addr = a_addr + Cfg::PART;
+#pragma unroll
+          for (int k = 0; k < Cfg::BK / Cfg::KMMA; ++k)
+            mma_pair<TF32>(d_tmem, smem_desc_sw128(a_addr + (uint32_t)k * a_step, a_lbo, a_sbo, a_mode),
+                           smem_desc_sw128(b_addr + (uint32_t)k * b_step, b_lbo, b_sbo, b_mode), idesc,
+                           (kb | k) != 0 ? 1u : 0u);
+          commit_pair(&empty_bar[stage]);
+          if (++stage == Cfg::STAGES) {
+            stage = 0;
+            phase ^= 1;
+          }
+        }
+        if (!ok) break;
+        commit_pair(&accf_bar[acc]);
+        if (++acc == 2) {
+          acc = 0;
+          acc_phase ^= 1;
+        }
+      }
+    }
+  } else {
+    const int quad = warp & 3, half = warp >> 2;
+    float* stage = reinterpret_cast<float*>(smem + Cfg::STAGES * Cfg::STAGE_BYTES) + warp * 32 * Cfg::STORE_COLS;
+    TileLoc L;
+    L.ldc = p.ldc; L.M = p.M; L.N = p.N; L.vecC = p.vecC; L.alpha = p.alpha; L.beta = p.beta;
+    int acc = 0;
+    uint32_t acc_phase = 0;
+    for (int tile = unit0; tile < p.num_tiles; tile += units) {
+      const bool ok = mbar_wait(&accf_bar[acc], acc_phase, p.status, kStatusTimeoutAcc);
+      if (!__all_sync(0xffffffffu, ok)) break;  // a warp's lanes go on, or give up, together
+      tc_fence_after();
+      int b, tm, tn;
+      tile_coords(p, tile, b, tm, tn);
+      const int row0 = tm * Cfg::BM + rank * Cfg::HALF + quad * 32;
+      float* cbase = p.C + (int64_t)b * p.strideC;
+      const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * Cfg::BN);
+#pragma unroll 1
+      for (int c0 = half * Cfg::HALF; c0 < (half + 1) * Cfg::HALF; c0 += 32) {
+        uint32_t r[32];
+        tmem_ld_32x32b_x32(tbase + (uint32_t)c0, r);
+        tmem_ld_wait();
+        if (row0 < p.M && tn * Cfg::BN + c0 < p.N)
+          store_chunk32<Cfg::STORE_COLS, true>(L, cbase, row0, tn * Cfg::BN + c0, stage, r, lane);
+        __syncwarp();
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) arrive_cluster(in_cta(smem_u32(&acce_bar[acc]), 0));
+      if (++acc == 2) {
+        acc = 0;
+        acc_phase ^= 1;
+      }
+    }
+  }
+
+  __syncthreads();
+  cluster_sync();  // neither CTA leaves while the other's loads, MMAs or arrivals may reach it
+  if (warp == Cfg::EPI_WARPS + 1) {
+    tc_fence_after();
+    tmem_dealloc_pair<Cfg::TMEM_COLS>(tmem_base);
   }
 }
 
