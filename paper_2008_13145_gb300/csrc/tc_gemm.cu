@@ -304,11 +304,17 @@ __global__ void prep_kernel(const PrepJob j) {
 template <typename TIn, typename TOut, bool SPLIT>
 __global__ void prep_group_kernel(const PrepJob* jobs, int n_jobs) {
   pdl_wait();
+  // The last job whose first block is not past this one: every lane looks at one of
+  // 32 evenly spaced jobs, then at one of those between two of them, so a hundred jobs
+  // take two dependent reads where a binary search took seven.
   const int blk = blockIdx.x;
-  int lo = 0, hi = n_jobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (jobs[mid].block_start <= blk) lo = mid; else hi = mid - 1;
+  int lo = 0, n = n_jobs;
+  while (n > 1) {
+    const int step = (n + 31) / 32, i = lo + (int)threadIdx.x * step;
+    const bool at = (int)threadIdx.x * step < n && jobs[i].block_start <= blk;
+    const int last = 31 - __clz(__ballot_sync(0xffffffffu, at));  // lane 0's job always qualifies
+    lo += last * step;
+    n = min(step, n - last * step);
   }
   const PrepJob j = jobs[lo];
   const int t = blk - j.block_start;

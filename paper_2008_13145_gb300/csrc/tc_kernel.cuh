@@ -125,15 +125,33 @@ struct TileLoc {
   float alpha, beta;
 };
 
+// First tiles of a group's problems, kept in shared memory: all of them for up
+// to kStarts problems, else every `step`-th.  Each role looks up each of its tiles;
+// eight dependent reads of descriptors in L2 (256 problems) held the loads back: the
+// grouped call of the 256-problem group took 421 us against 386 so.
+constexpr int kStarts = 448;
+struct GroupIndex {
+  const int* starts;
+  int n, step;
+};
+
 template <bool GROUPED>
-__device__ __forceinline__ TileLoc locate(const TcArgs& p, const GroupArgs& g, const CUtensorMap* ma,
-                                          const CUtensorMap* mb, int tile) {
+__device__ __forceinline__ TileLoc locate(const TcArgs& p, const GroupArgs& g, const GroupIndex& x,
+                                          const CUtensorMap* ma, const CUtensorMap* mb, int tile) {
   TileLoc L;
   if constexpr (GROUPED) {
-    int lo = 0, hi = g.count - 1;  // last problem whose tile_start <= tile
+    int lo = 0, hi = x.n - 1;  // last problem whose tile_start <= tile
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (g.descs[mid].tile_start <= tile) lo = mid; else hi = mid - 1;
+      if (x.starts[mid] <= tile) lo = mid; else hi = mid - 1;
+    }
+    if (x.step > 1) {
+      lo *= x.step;
+      hi = min(lo + x.step, g.count) - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (g.descs[mid].tile_start <= tile) lo = mid; else hi = mid - 1;
+      }
     }
     const GroupDesc& d = g.descs[lo];
     const int t = tile - d.tile_start;
@@ -286,6 +304,14 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, TF32>::THREADS, 1)
   // memory, so it may overlap the previous kernel's tail.
   pdl_wait();
   pdl_launch_dependents();
+  __shared__ int starts_sh[GROUPED ? kStarts : 1];
+  GroupIndex index{starts_sh, 0, 1};
+  if constexpr (GROUPED) {
+    index.step = (g.count + kStarts - 1) / kStarts;
+    index.n = (g.count + index.step - 1) / index.step;
+    for (int i = threadIdx.x; i < index.n; i += Cfg::THREADS) starts_sh[i] = g.descs[i * index.step].tile_start;
+    __syncthreads();
+  }
 
   if (warp == Cfg::EPI_WARPS) {
     // ---------------------------------------------------------------- TMA producer
@@ -294,7 +320,7 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, TF32>::THREADS, 1)
       uint32_t phase = 0;
       bool ok = true;
       for (int tile = unit0; tile < p.num_tiles && ok; tile += units) {
-        const TileLoc L = locate<GROUPED>(p, g, &tmA, &tmB, tile);
+        const TileLoc L = locate<GROUPED>(p, g, index, &tmA, &tmB, tile);
         for (int kb = 0; kb < L.k_blocks; ++kb) {
           if (!(ok = mbar_wait(&empty_bar[stage], phase ^ 1, p.status, kStatusTimeoutEmpty))) break;
           uint8_t* sa = smem + stage * Cfg::STAGE_BYTES;
@@ -351,7 +377,7 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, TF32>::THREADS, 1)
       for (int tile = unit0; tile < p.num_tiles && ok; tile += units) {
         int k_blocks = p.k_blocks, a_mn = p.a_mn, b_mn = p.b_mn;
         if constexpr (GROUPED) {
-          const TileLoc L = locate<true>(p, g, &tmA, &tmB, tile);
+          const TileLoc L = locate<true>(p, g, index, &tmA, &tmB, tile);
           k_blocks = L.k_blocks;
           a_mn = L.a_mn;
           b_mn = L.b_mn;
@@ -400,7 +426,7 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, TF32>::THREADS, 1)
     for (int tile = unit0; tile < p.num_tiles; tile += units) {
       if (!mbar_wait(&accf_bar[acc], acc_phase, p.status, kStatusTimeoutAcc)) break;
       tc_fence_after();
-      const TileLoc L = locate<GROUPED>(p, g, &tmA, &tmB, tile);
+      const TileLoc L = locate<GROUPED>(p, g, index, &tmA, &tmB, tile);
       const int quad = warp & 3, row0 = L.tm * kBM + quad * 32;
       constexpr int COLS = BN / (Cfg::EPI_WARPS / 4);  // columns of this warp
       const int col0 = (warp >> 2) * COLS;
