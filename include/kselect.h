@@ -615,6 +615,18 @@ gemm_status_t select_kernels_batched(gemm_handle_t handle, int32_t n, const int6
 gemm_status_t kselect_im2col3x3(const float* x_dev, int32_t N, int32_t H, int32_t W, int32_t C, float* out_dev,
                                 int64_t ld, void* stream);
 
+/* out (N*H*W rows of Cout) = max(0, conv3x3(x) + bias): the product of x's
+ * neighbourhoods (kselect_im2col3x3) and the weights (Cout x 9 C, op(B) = B^T)
+ * with the kernel the handle selects for those sizes, as the three calls
+ * kselect_im2col3x3, gemm and kselect_bias_act give it (bias may be NULL, relu
+ * 0).  Where C is a multiple of 32 and the tensor cores run the product at FP32
+ * accuracy (see gemm), they read the image itself and add bias and ReLU as they
+ * store; otherwise `col` (N*H*W rows of ld >= 9 C floats) receives the
+ * neighbourhoods, and may not be NULL. */
+gemm_status_t kselect_conv3x3(gemm_handle_t handle, const float* x_dev, int32_t N, int32_t H, int32_t W, int32_t C,
+                              const float* weights_dev, int32_t Cout, const float* bias_dev, int32_t relu,
+                              float* col_dev, int64_t ld, float* out_dev, void* stream);
+
 /* y[r, j] = y[r, j] + bias[j] (bias may be NULL), then max(., 0) if relu. */
 gemm_status_t kselect_bias_act(float* y_dev, int64_t rows, int32_t cols, int64_t ld, const float* bias_dev,
                                int32_t relu, void* stream);

@@ -99,6 +99,15 @@ __device__ __forceinline__ bool ks_in_bounds(const GemmArgs& p, int op, const vo
   return true;
 }
 
+// A 3 x 3 convolution (padding 1) of an NHWC image as the A of a product:
+// M = images x H x W, K = 9 C, C a multiple of 32, 16-byte aligned.  bias (N
+// values, or null) and relu apply to the result; with split K the caller adds them.
+struct Conv3x3 {
+  int H, W, C;
+  const float* bias;
+  int relu;
+};
+
 using LaunchFn = cudaError_t (*)(const GemmArgs&, cudaStream_t);
 using OccFn = int (*)();  // resident CTAs per SM on the current device, 0 on error
 

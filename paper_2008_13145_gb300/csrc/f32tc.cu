@@ -87,7 +87,15 @@ struct Args {
   int group_m;
   int vec8;  // C takes 32-byte stores
   int* status;
+  // 3 x 3 convolution (kConv): A is the NHWC image; bias and ReLU go with the stores.
+  int H, W, Ch;
+  const float* bias;  // N values or null
+  int relu;
 };
+
+// How A reaches the kernel: stored with K contiguous, with M contiguous, or as
+// the image that its rows are the 3 x 3 neighbourhoods of.
+enum : int { kRows = 0, kCols = 1, kConv = 2 };
 
 // Tile row (or column) r of an R-wide operand slice sits in shared-memory row
 // (r % 4) * (R / 4) + r / 4.  A thread that loads four consecutive elements
@@ -123,8 +131,8 @@ __device__ __forceinline__ void sts64(uint32_t addr, uint32_t x, uint32_t y) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(x), "r"(y) : "memory");
 }
 // One operand's slice of R rows (M of A, N of B) x 32 K as this thread loads and
-// stores it.  MN: stored with R contiguous; otherwise K contiguous.
-template <int R, bool MN>
+// stores it.
+template <int R, int KIND>
 struct Slice;
 
 // The slice is stored and the next one loaded part by part (`parts` of them),
@@ -133,7 +141,7 @@ struct Slice;
 // K contiguous: a warp instruction covers 4 rows x 128 bytes of K; part t is 4
 // consecutive K of one row.  Warp w of the group has rows w, w + 4, ...
 template <int R>
-struct Slice<R, false> {
+struct Slice<R, kRows> {
   static constexpr int PARTS = R / 16, N = 4;
   const float* ptr;  // (row of part 0, K) of the chunk to load
   int64_t step;      // 16 rows on
@@ -143,7 +151,7 @@ struct Slice<R, false> {
     sm = warp * (R / 4) + (lane >> 3);
     kq = lane & 7;
   }
-  __device__ __forceinline__ void start(const float* base, int64_t ld, int r0, int rows, int k0) {
+  __device__ __forceinline__ void start(const Args&, const float* base, int64_t ld, int r0, int rows, int k0) {
     lim = rows - r0 - row;  // part t's row exists when 16 t < lim
     ptr = base + (int64_t)(r0 + row) * ld + k0 + 4 * kq;
     step = 16 * ld;
@@ -174,7 +182,7 @@ struct Slice<R, false> {
 // R contiguous: part t is 4 consecutive rows x 4 consecutive K; a warp's part
 // covers 32 rows x 16 K, each of its loads 4 K rows x 128 bytes.
 template <int R>
-struct Slice<R, true> {
+struct Slice<R, kCols> {
   static constexpr int PARTS = R / 64, N = 16;
   const float* ptr;
   int64_t ld;
@@ -185,7 +193,7 @@ struct Slice<R, true> {
     row = 4 * sm;
     k = 16 * (warp / MB) + 4 * ((lane & 1) | ((lane >> 3) & 2));
   }
-  __device__ __forceinline__ void start(const float* base, int64_t ld_, int r0, int rows, int k0) {
+  __device__ __forceinline__ void start(const Args&, const float* base, int64_t ld_, int r0, int rows, int k0) {
     ld = ld_;
     lim = rows - r0 - row;  // rows that exist of this thread's 4
     ptr = base + (int64_t)(k0 + k) * ld + r0 + row;
@@ -215,6 +223,58 @@ struct Slice<R, true> {
 #pragma unroll
       for (int s = 0; s < kParts; ++s) sts64(at + s * (R * 64), x[s], y[s]);
     }
+  }
+};
+
+// Neighbourhoods of an NHWC image with a multiple of 32 channels: column
+// (kh * 3 + kw) * Ch + c of row (n, h, w) is x[n, h + kh - 1, w + kw - 1, c], zero
+// outside.  A chunk then lies in one tap, and moving a tap on moves every row's
+// address by the same distance, so this is the K-contiguous slice with rows of
+// Ch, plus one bit per row and tap that says whether the tap is inside.  (Written
+// out by a separate pass, the neighbourhoods are nine times the image: 1.64 of
+// the 5.06 ms of VGG16 on 16 images.)
+template <int R>
+struct Slice<R, kConv> : Slice<R, kRows> {
+  using Base = Slice<R, kRows>;
+  using Base::N;
+  using Base::PARTS;
+  uint32_t inside[(PARTS + 2) / 3];  // nine bits a part, three parts a word
+  int c, tap;
+  int64_t down;  // from the end of a tap's channels to the next row of taps
+  int channels;
+  __device__ __forceinline__ void start(const Args& p, const float* x, int64_t, int r0, int rows, int k0) {
+    channels = p.Ch;
+    tap = k0 / p.Ch;
+    c = k0 - tap * p.Ch;
+    down = (int64_t)(p.W - 3) * p.Ch;
+    this->step = 16 * (int64_t)p.Ch;
+    this->ptr = x + ((int64_t)(r0 + this->row) + (tap / 3 - 1) * p.W + (tap % 3 - 1)) * p.Ch + c + 4 * this->kq;
+#pragma unroll
+    for (int i = 0; i < (PARTS + 2) / 3; ++i) inside[i] = 0;
+#pragma unroll
+    for (int t = 0; t < PARTS; ++t) {
+      const int m = r0 + this->row + 16 * t, hw = m % (p.H * p.W), h = hw / p.W, w = hw - h * p.W;
+      uint32_t in = 0;
+      if (m < rows) {
+        const uint32_t cols = (w > 0 ? 1u : 0u) | 2u | (w + 1 < p.W ? 4u : 0u);
+        in = (h > 0 ? cols : 0u) | cols << 3 | (h + 1 < p.H ? cols << 6 : 0u);
+      }
+      inside[t / 3] |= in << (9 * (t % 3));
+    }
+  }
+  __device__ __forceinline__ void advance() {
+    this->ptr += kBK;
+    c += kBK;
+    if (c == channels) {
+      c = 0;
+      if (++tap % 3 == 0) this->ptr += down;
+    }
+  }
+  __device__ __forceinline__ void load(int t, float (&v)[N], bool, bool, int) const {
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if ((inside[t / 3] >> (9 * (t % 3) + tap)) & 1)
+      x = __ldg(reinterpret_cast<const float4*>(this->ptr + t * this->step));
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
   }
 };
 
@@ -290,8 +350,20 @@ __device__ __forceinline__ void issue_mmas(uint32_t a0, uint32_t d, uint64_t* sl
   mma_commit(acc_full);
 }
 
-// Up to four (`left`) consecutive columns of one row of C.
-__device__ __forceinline__ void store4(const GemmArgs& g, float* dst, int left, const float (&v)[4]) {
+// Bias and ReLU of column n, where the launch has them.
+template <bool ACT>
+__device__ __forceinline__ float act(const Args& p, int n, float v) {
+  if constexpr (ACT) {
+    if (p.bias) v += __ldg(p.bias + n);
+    if (p.relu) v = fmaxf(v, 0.f);
+  }
+  return v;
+}
+
+// Up to four (`left`) consecutive columns of one row of C, from column n on.
+template <bool ACT>
+__device__ __forceinline__ void store4(const Args& p, float* dst, int n, int left, const float (&v)[4]) {
+  const GemmArgs& g = p.g;
   float o[4] = {g.alpha * v[0], g.alpha * v[1], g.alpha * v[2], g.alpha * v[3]};
   if (g.vecC && left >= 4) {
     if (g.beta != 0.f) {
@@ -299,11 +371,12 @@ __device__ __forceinline__ void store4(const GemmArgs& g, float* dst, int left, 
       o[0] = fmaf(g.beta, c.x, o[0]); o[1] = fmaf(g.beta, c.y, o[1]);
       o[2] = fmaf(g.beta, c.z, o[2]); o[3] = fmaf(g.beta, c.w, o[3]);
     }
-    *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+    *reinterpret_cast<float4*>(dst) =
+        make_float4(act<ACT>(p, n, o[0]), act<ACT>(p, n + 1, o[1]), act<ACT>(p, n + 2, o[2]), act<ACT>(p, n + 3, o[3]));
   } else {
 #pragma unroll
     for (int e = 0; e < 4; ++e)
-      if (e < left) dst[e] = g.beta != 0.f ? fmaf(g.beta, dst[e], o[e]) : o[e];
+      if (e < left) dst[e] = act<ACT>(p, n + e, g.beta != 0.f ? fmaf(g.beta, dst[e], o[e]) : o[e]);
   }
 }
 
@@ -314,7 +387,7 @@ __device__ __forceinline__ void store4(const GemmArgs& g, float* dst, int left, 
 // of bank conflicts both ways) and leave as 64-byte runs of a row: lanes
 // writing 4 bytes of 32 different rows took 109 us against 34 (SIMT kernel) at
 // 1433 x 2406 x 18 x 16 with odd rows.
-template <int G>
+template <int G, bool ACT>
 __device__ __forceinline__ void store_rows(const Args& p, const Item& it, int row0, int col, const float (&acc)[4][G],
                                            uint32_t stage, int lane) {
   const float alpha = p.g.alpha, beta = p.g.beta;
@@ -335,6 +408,8 @@ __device__ __forceinline__ void store_rows(const Args& p, const Item& it, int ro
         o[4] = fmaf(beta, c1.x, o[4]); o[5] = fmaf(beta, c1.y, o[5]);
         o[6] = fmaf(beta, c1.z, o[6]); o[7] = fmaf(beta, c1.w, o[7]);
       }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[e] = act<ACT>(p, col + 4 * q + e, o[e]);
       asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(o[0]), "f"(o[1]),
                    "f"(o[2]), "f"(o[3]), "f"(o[4]), "f"(o[5]), "f"(o[6]), "f"(o[7])
                    : "memory");
@@ -362,7 +437,8 @@ __device__ __forceinline__ void store_rows(const Args& p, const Item& it, int ro
                      : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3])
                      : "r"(stage + r * 64 + (((lane & 3) ^ ((r >> 1) & 3)) << 4))
                      : "memory");
-        if (row < p.g.M && c < left) store4(p.g, base + (int64_t)row * p.g.ldc + 16 * blk + c, left - c, o);
+        if (row < p.g.M && c < left)
+          store4<ACT>(p, base + (int64_t)row * p.g.ldc + 16 * blk + c, col + 16 * blk + c, left - c, o);
       }
     } else {
 #pragma unroll 4
@@ -376,7 +452,7 @@ __device__ __forceinline__ void store_rows(const Args& p, const Item& it, int ro
         if (row < p.g.M && c < left) {
           float* dst = base + (int64_t)row * p.g.ldc + 16 * blk + c;
           o *= alpha;
-          *dst = beta != 0.f ? fmaf(beta, *dst, o) : o;
+          *dst = act<ACT>(p, col + 16 * blk + c, beta != 0.f ? fmaf(beta, *dst, o) : o);
         }
       }
     }
@@ -384,14 +460,22 @@ __device__ __forceinline__ void store_rows(const Args& p, const Item& it, int ro
 }
 
 // `quads` groups of four columns of one row of an item by plain FP32 FMAs over
-// its K range, in K order (out of line: the tiles that need it are rare).
-template <bool A_MN, bool B_MN>
-__device__ __forceinline__ void redo_row(const GemmArgs& g, const Item& it, int row, int col, int quads) {
+// its K range, in K order.
+template <int AK, bool B_MN>
+__device__ __forceinline__ void redo_row(const Args& p, const Item& it, int row, int col, int quads) {
+  const GemmArgs& g = p.g;
   if (row >= g.M) return;
-  const float* A = static_cast<const float*>(g.A) + (int64_t)it.b * g.strideA + (A_MN ? (int64_t)row : row * g.lda);
+  const float* A = static_cast<const float*>(g.A) + (int64_t)it.b * g.strideA +
+                   (AK == kCols ? (int64_t)row : row * g.lda);
   const float* B = static_cast<const float*>(g.B) + (int64_t)it.b * g.strideB;
   float* crow = g.C + it.slab * g.strideC + (int64_t)row * g.ldc;
-  const int64_t as = A_MN ? g.lda : 1, bk = B_MN ? g.ldb : 1, bn = B_MN ? 1 : g.ldb;
+  const int64_t as = AK == kCols ? g.lda : 1, bk = B_MN ? g.ldb : 1, bn = B_MN ? 1 : g.ldb;
+  int h = 0, w = 0;
+  if constexpr (AK == kConv) {
+    const int hw = row % (p.H * p.W);
+    h = hw / p.W;
+    w = hw - h * p.W;
+  }
 #pragma unroll 1
   for (int q = 0; q < quads; ++q) {
     const int n = col + 4 * q;
@@ -402,15 +486,22 @@ __device__ __forceinline__ void redo_row(const GemmArgs& g, const Item& it, int 
     float v[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
     for (int k = it.kbeg; k < it.kend; ++k) {
-      const float a = __ldg(A + k * as);
+      float a;
+      if constexpr (AK == kConv) {
+        const int tap = k / p.Ch, dh = tap / 3 - 1, dw = tap % 3 - 1;
+        const bool in = (unsigned)(h + dh) < (unsigned)p.H && (unsigned)(w + dw) < (unsigned)p.W;
+        a = in ? __ldg(A + (int64_t)(dh * p.W + dw) * p.Ch + (k - tap * p.Ch)) : 0.f;
+      } else {
+        a = __ldg(A + k * as);
+      }
 #pragma unroll
       for (int e = 0; e < 4; ++e) v[e] = fmaf(a, __ldg(b[e] + k * bk), v[e]);
     }
-    store4(g, crow + n, g.N - n, v);
+    store4<AK == kConv>(p, crow + n, n, g.N - n, v);
   }
 }
 
-template <int BN, bool A_MN, bool B_MN>
+template <int BN, int AK, bool B_MN>
 __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constant__ Args p) {
   using C = Cfg<BN>;
   constexpr int G = C::G;
@@ -458,8 +549,8 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
     // ---------------------------------------------------------------- load and convert
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::REGS_CONVERT));
     const int group = (warp - kReaders) >> 2;
-    using SA = Slice<kBM, A_MN>;
-    using SB = Slice<BN, B_MN>;
+    using SA = Slice<kBM, AK>;
+    using SB = Slice<BN, B_MN ? kCols : kRows>;
     SA sa;
     SB sb;
     sa.place(warp & 3, lane);
@@ -470,8 +561,8 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
     auto next_item = [&]() {
       item += gridDim.x;
       const Item it = item_of<BN>(p, item);
-      sa.start(static_cast<const float*>(p.g.A) + (int64_t)it.b * p.g.strideA, p.g.lda, it.m0, p.g.M, it.kbeg);
-      sb.start(static_cast<const float*>(p.g.B) + (int64_t)it.b * p.g.strideB, p.g.ldb, it.n0, p.g.N, it.kbeg);
+      sa.start(p, static_cast<const float*>(p.g.A) + (int64_t)it.b * p.g.strideA, p.g.lda, it.m0, p.g.M, it.kbeg);
+      sb.start(p, static_cast<const float*>(p.g.B) + (int64_t)it.b * p.g.strideB, p.g.ldb, it.n0, p.g.N, it.kbeg);
       left = it.kend - it.kbeg;
       fa = p.g.vecA && it.m0 + kBM <= p.g.M;
       fb = p.g.vecB && it.n0 + BN <= p.g.N;
@@ -573,8 +664,8 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
       for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int q = 0; q < G; ++q) lost |= !(fabsf(acc[j][q]) <= 3.402823466e38f);
-      if (__any_sync(0xffffffffu, lost)) redo_row<A_MN, B_MN>(p.g, it, row0 + 4 * lane, col, G);
-      else store_rows<G>(p, it, row0, col, acc, stage, lane);
+      if (__any_sync(0xffffffffu, lost)) redo_row<AK, B_MN>(p, it, row0 + 4 * lane, col, G);
+      else store_rows<G, AK == kConv>(p, it, row0, col, acc, stage, lane);
     }
   }
   __syncthreads();
@@ -584,9 +675,9 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
   }
 }
 
-template <int BN, bool A_MN, bool B_MN>
+template <int BN, int AK, bool B_MN>
 cudaError_t launch(const Args& a, int sms, cudaStream_t s) {
-  auto kern = f32tc_kernel<BN, A_MN, B_MN>;
+  auto kern = f32tc_kernel<BN, AK, B_MN>;
   static unsigned long long done_mask = 0;  // devices whose attribute is set
   int dev = 0;
   cudaGetDevice(&dev);
@@ -605,9 +696,10 @@ cudaError_t launch(const Args& a, int sms, cudaStream_t s) {
 
 template <int BN>
 cudaError_t launch_bn(const Args& a, int sms, cudaStream_t s) {
-  const bool am = a.g.transA != 0, bm = a.g.transB == 0;
-  if (am) return bm ? launch<BN, true, true>(a, sms, s) : launch<BN, true, false>(a, sms, s);
-  return bm ? launch<BN, false, true>(a, sms, s) : launch<BN, false, false>(a, sms, s);
+  const bool bm = a.g.transB == 0;
+  if (a.Ch > 0) return launch<BN, kConv, false>(a, sms, s);
+  if (a.g.transA) return bm ? launch<BN, kCols, true>(a, sms, s) : launch<BN, kCols, false>(a, sms, s);
+  return bm ? launch<BN, kRows, true>(a, sms, s) : launch<BN, kRows, false>(a, sms, s);
 }
 
 // ---------------------------------------------------------------- two CTAs on one 256 x 256 tile
@@ -649,7 +741,7 @@ __device__ __forceinline__ void convert_pair(const Args& p, int total, bool is_a
     const int r0 = (is_a ? it.m0 : it.n0) + 128 * (int)rank, rows = is_a ? p.g.M : p.g.N;
     const float* base = static_cast<const float*>(is_a ? p.g.A : p.g.B) +
                         (int64_t)it.b * (is_a ? p.g.strideA : p.g.strideB);
-    sl.start(base, is_a ? p.g.lda : p.g.ldb, r0, rows, it.kbeg);
+    sl.start(p, base, is_a ? p.g.lda : p.g.ldb, r0, rows, it.kbeg);
     left = it.kend - it.kbeg;
     inner = vec && r0 + 128 <= rows;
   };
@@ -699,7 +791,7 @@ __device__ __forceinline__ void convert_pair(const Args& p, int total, bool is_a
   }
 }
 
-template <bool A_MN, bool B_MN>
+template <int AK, bool B_MN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     f32tc_pair_kernel(const __grid_constant__ Args p) {
   constexpr int G = Pair::G;
@@ -759,8 +851,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   } else if (warp >= kReaders) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPairRegsConvert));
-    if (warp < kReaders + 4) convert_pair<Slice<128, A_MN>>(p, total, true, rank, smem, full, empty, inexact, warp, lane);
-    else convert_pair<Slice<128, B_MN>>(p, total, false, rank, smem, full, empty, inexact, warp, lane);
+    if (warp < kReaders + 4) convert_pair<Slice<128, AK>>(p, total, true, rank, smem, full, empty, inexact, warp, lane);
+    else convert_pair<Slice<128, B_MN ? kCols : kRows>>(p, total, false, rank, smem, full, empty, inexact, warp, lane);
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPairRegsRead));
     float acc[4][G];
@@ -805,8 +897,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int q = 0; q < G; ++q) lost |= !(fabsf(acc[j][q]) <= 3.402823466e38f);
-      if (__any_sync(0xffffffffu, lost)) redo_row<A_MN, B_MN>(p.g, it, row0 + 4 * lane, col, G);
-      else store_rows<G>(p, it, row0, col, acc, stage, lane);
+      if (__any_sync(0xffffffffu, lost)) redo_row<AK, B_MN>(p, it, row0 + 4 * lane, col, G);
+      else store_rows<G, AK == kConv>(p, it, row0, col, acc, stage, lane);
     }
   }
   __syncthreads();
@@ -817,9 +909,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   }
 }
 
-template <bool A_MN, bool B_MN>
+template <int AK, bool B_MN>
 cudaError_t launch_pair(const Args& a, int sms, cudaStream_t s) {
-  auto kern = f32tc_pair_kernel<A_MN, B_MN>;
+  auto kern = f32tc_pair_kernel<AK, B_MN>;
   static unsigned long long done_mask = 0;
   int dev = 0;
   cudaGetDevice(&dev);
@@ -842,8 +934,19 @@ cudaError_t launch_pair(const Args& a, int sms, cudaStream_t s) {
 // Runs the kernel with BN-wide tiles.  With splits > 1, `g` describes the
 // workspace of partial products (alpha 1, beta 0, one M x ldc slab per batch
 // entry and split, strideC apart), split s covering K [s * kchunk, (s + 1) * kchunk).
-cudaError_t f32tc_launch(int bn, const GemmArgs& g, int splits, int kchunk, int sms, int* status, cudaStream_t s) {
+// `conv`: A is an NHWC image and M = its positions, K = 9 x its channels (see Conv3x3).
+cudaError_t f32tc_launch(int bn, const GemmArgs& g, int splits, int kchunk, int sms, int* status, cudaStream_t s,
+                         const Conv3x3* conv) {
   f32tc::Args a;
+  a.H = a.W = a.Ch = a.relu = 0;
+  a.bias = nullptr;
+  if (conv) {
+    a.H = conv->H;
+    a.W = conv->W;
+    a.Ch = conv->C;
+    a.bias = conv->bias;
+    a.relu = conv->relu;
+  }
   a.g = g;
   const int bm = bn == 256 ? 256 : f32tc::kBM;
   a.tiles_m = (g.M + bm - 1) / bm;
@@ -858,9 +961,11 @@ cudaError_t f32tc_launch(int bn, const GemmArgs& g, int splits, int kchunk, int 
   if (bn == 64) return f32tc::launch_bn<64>(a, sms, s);
   if (bn == 128) return f32tc::launch_bn<128>(a, sms, s);
   if (bn == 256) {
-    const bool am = g.transA != 0, bmn = g.transB == 0;
-    if (am) return bmn ? f32tc::launch_pair<true, true>(a, sms, s) : f32tc::launch_pair<true, false>(a, sms, s);
-    return bmn ? f32tc::launch_pair<false, true>(a, sms, s) : f32tc::launch_pair<false, false>(a, sms, s);
+    using namespace f32tc;
+    const bool bmn = g.transB == 0;
+    if (a.Ch > 0) return launch_pair<kConv, false>(a, sms, s);
+    if (g.transA) return bmn ? launch_pair<kCols, true>(a, sms, s) : launch_pair<kCols, false>(a, sms, s);
+    return bmn ? launch_pair<kRows, true>(a, sms, s) : launch_pair<kRows, false>(a, sms, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -359,7 +359,8 @@ static gemm_status_t launch_split(int base, const GemmArgs& a, int splits, int k
 }
 
 // ------------------------------------------------------------------ FP32 on the tensor cores (f32tc.cu)
-cudaError_t f32tc_launch(int bn, const GemmArgs& g, int splits, int kchunk, int sms, int* status, cudaStream_t s);
+cudaError_t f32tc_launch(int bn, const GemmArgs& g, int splits, int kchunk, int sms, int* status, cudaStream_t s,
+                         const Conv3x3* conv);
 int* tc_status_word();
 int* tc_status_word_if_ready();
 
@@ -438,20 +439,12 @@ static double simt_cost(int id, const GemmArgs& a, int dev, int sms, int* splits
   return us;
 }
 
-// Whether an FP32 request for which SIMT kernel `id` was selected runs on the
-// tensor cores, and how.  Split factors tried: those that fill one round and two
-// rounds of CTAs, since the model's cost falls with the K range of an item and
-// rises with the rounds (this runs on every call, so it stays short).
-static bool f32tc_plan(int id, const GemmArgs& a, int dev, int sms, F32tcPlan* plan) {
-  if (a.K < kF32tcMinK || sms < 2) return false;
-  const double outputs = (double)a.M * (double)a.N * (double)a.batch;
-  if (outputs > 1e12) return false;  // keeps the tile counts small
-  if (2.0 * outputs * a.K < kF32tcMinFlops) return false;
-  int simt_splits = 1;
-  double best = simt_cost(id, a, dev, sms, &simt_splits);
-  if (best < kF32tcMinSimtUs) return false;
-  best /= kF32tcMargin;
-  const double error = 0.9 * simt_error(a.K, simt_splits);
+// The fastest way to run an FP32 product on the tensor cores that the model
+// puts below `limit_us` and below `limit_error`.  Split factors tried: none, and
+// those that just fill one to four rounds of CTAs, since the model's cost falls
+// with the K range of an item and rises with the rounds (this runs on every
+// call, so it stays short).
+static bool f32tc_fastest(const GemmArgs& a, int sms, double limit_us, double limit_error, F32tcPlan* plan) {
   bool found = false;
   const int nk = (a.K + kF32tcChunk - 1) / kF32tcChunk;
   const int64_t slab = (int64_t)a.batch * a.M * (((int64_t)a.N + 7) / 8 * 8) * 4;
@@ -459,7 +452,7 @@ static bool f32tc_plan(int id, const GemmArgs& a, int dev, int sms, F32tcPlan* p
     const int bm = c.bn == 256 ? 256 : 128, units = c.bn == 256 ? sms / 2 : sms;
     const int64_t tiles = ceil_div(a.M, bm) * ceil_div(a.N, c.bn) * a.batch;
     int last = 0;
-    for (int rounds = 0; rounds <= 2; ++rounds) {
+    for (int rounds = 0; rounds <= 4; ++rounds) {
       int S = rounds == 0 ? 1 : (int)std::min<int64_t>(rounds * units / tiles, std::min(kSplitMaxFactor, nk / 2));
       if (S <= last) continue;
       const int kc = (nk + S - 1) / S;
@@ -467,10 +460,10 @@ static bool f32tc_plan(int id, const GemmArgs& a, int dev, int sms, F32tcPlan* p
       if (S <= last) continue;
       last = S;
       if (S > 1 && S * slab > kSplitWorkspaceMax) break;
-      if (f32tc_error(a.K, S) > error) continue;
+      if (f32tc_error(a.K, S) > limit_error) continue;
       const double us = f32tc_cost(c, a, tiles, kc, S, units);
-      if (us < best) {
-        best = us;
+      if (us < limit_us) {
+        limit_us = us;
         found = true;
         *plan = F32tcPlan{c.bn, S, kc * kF32tcChunk};
       }
@@ -479,11 +472,25 @@ static bool f32tc_plan(int id, const GemmArgs& a, int dev, int sms, F32tcPlan* p
   return found;
 }
 
-static gemm_status_t f32tc_run(const F32tcPlan& plan, const GemmArgs& a, int sms, int* status, cudaStream_t s) {
+// Whether an FP32 request for which SIMT kernel `id` was selected runs on the
+// tensor cores, and how; other_us: what else the SIMT kernel would need first.
+static bool f32tc_plan(int id, const GemmArgs& a, int dev, int sms, double other_us, F32tcPlan* plan) {
+  if (a.K < kF32tcMinK || sms < 2) return false;
+  const double outputs = (double)a.M * (double)a.N * (double)a.batch;
+  if (outputs > 1e12) return false;  // keeps the tile counts small
+  if (2.0 * outputs * a.K < kF32tcMinFlops) return false;
+  int simt_splits = 1;
+  const double us = simt_cost(id, a, dev, sms, &simt_splits) + other_us;
+  if (us < kF32tcMinSimtUs) return false;
+  return f32tc_fastest(a, sms, us / kF32tcMargin, 0.9 * simt_error(a.K, simt_splits), plan);
+}
+
+static gemm_status_t f32tc_run(const F32tcPlan& plan, const GemmArgs& a, int sms, int* status, cudaStream_t s,
+                               const Conv3x3* conv = nullptr) {
   const int bn = plan.bn, splits = plan.splits, kchunk = plan.kchunk;
   cudaError_t e;
   if (splits <= 1) {
-    e = f32tc_launch(bn, a, 1, a.K, sms, status, s);
+    e = f32tc_launch(bn, a, 1, a.K, sms, status, s, conv);
     if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
     return GEMM_OK;
   }
@@ -498,7 +505,7 @@ static gemm_status_t f32tc_run(const F32tcPlan& plan, const GemmArgs& a, int sms
   p.ldc = ldw;
   p.strideC = ldw * a.M;
   p.vecC = 1;
-  e = f32tc_launch(bn, p, splits, kchunk, sms, status, s);
+  e = f32tc_launch(bn, p, splits, kchunk, sms, status, s, conv);
   if (e == cudaSuccess) {
     const int64_t total = (int64_t)a.batch * a.M * ((a.N + 3) / 4);
     const int grid = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
@@ -556,6 +563,14 @@ static gemm_status_t launch_config(int id, const GemmArgs& a, cudaStream_t s) {
   return GEMM_ERR_NO_KERNEL;
 }
 
+// The device's tensor-core status word; null where it would have to be made while `s` is captured.
+static int* status_word_for(cudaStream_t s) {
+  if (int* w = tc_status_word_if_ready()) return w;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return nullptr;
+  return tc_status_word();
+}
+
 // Runs the kernel a handle selected.  A SIMT choice is run on the tensor cores
 // at FP32 accuracy (f32tc.cu: closer to the exact product than the SIMT kernels'
 // FMA chains) where that is expected to be faster.  The device's first
@@ -566,14 +581,9 @@ static gemm_status_t launch_selected(int id, const GemmArgs& a, cudaStream_t s) 
   if (cudaGetDevice(&dev) != cudaSuccess) return launch_config(id, a, s);
   const int sms = sm_count_of(dev);
   F32tcPlan plan;
-  if (!f32tc_plan(id, a, dev, sms, &plan)) return launch_config(id, a, s);
-  int* status = tc_status_word_if_ready();
-  if (!status) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
-      return launch_config(id, a, s);
-    if (!(status = tc_status_word())) return launch_config(id, a, s);
-  }
+  if (!f32tc_plan(id, a, dev, sms, 0.0, &plan)) return launch_config(id, a, s);
+  int* status = status_word_for(s);
+  if (!status) return launch_config(id, a, s);
   return f32tc_run(plan, a, sms, status, s);
 }
 
@@ -897,6 +907,47 @@ gemm_status_t gemm(gemm_handle_t h, char transA, char transB, int64_t M, int64_t
   return launch_selected(id, a, static_cast<cudaStream_t>(stream));
 }
 
+gemm_status_t kselect_conv3x3(gemm_handle_t h, const float* x, int32_t N, int32_t H, int32_t W, int32_t C,
+                              const float* weights, int32_t Cout, const float* bias, int32_t relu, float* col,
+                              int64_t ld, float* out, void* stream) {
+  if (!h || N < 0 || H < 0 || W < 0 || C < 1 || Cout < 0 || ld < 9LL * C) return GEMM_ERR_INVALID_ARG;
+  const int64_t M = (int64_t)N * H * W, K = 9LL * C;
+  if (M == 0 || Cout == 0) return GEMM_OK;
+  if (!x || !weights || !out) return GEMM_ERR_INVALID_ARG;
+  const int32_t id = select_kernel(h, M, Cout, K, 1);
+  if (id < 0) return (gemm_status_t)id;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  // FP32 classes, channels in whole K chunks, 16-byte rows: straight from the image.
+  const int fam = family_of(id);
+  GemmArgs a;
+  bool noop = false;
+  int dev = 0;
+  if ((fam == GEMM_PREC_F32 || fam == GEMM_PREC_F32X3) && C % 32 == 0 && (uintptr_t)x % 16 == 0 &&
+      (uintptr_t)weights % 16 == 0 && cudaGetDevice(&dev) == cudaSuccess &&
+      make_args('N', 'T', M, Cout, K, 1.f, x, K, weights, K, 0.f, out, Cout, 1, 4, &a, &noop) == GEMM_OK && !noop) {
+    a.lda = C;  // of the image; its neighbourhoods are not stored
+    const int sms = sm_count_of(dev);
+    const double col_us = 2e6 * M * K * 4 / kSplitReduceBps;  // writing the neighbourhoods out and reading them back
+    F32tcPlan plan;
+    // A split-BF16 choice is less exact, and needs the neighbourhoods split as well: it never stays ahead.
+    const bool use = fam == GEMM_PREC_F32 ? f32tc_plan(id, a, dev, sms, col_us, &plan)
+                                          : (double)M * Cout < 1e12 && 2.0 * M * Cout * K >= kF32tcMinFlops &&
+                                                sms >= 2 && f32tc_fastest(a, sms, INFINITY, INFINITY, &plan);
+    int* status = use ? status_word_for(s) : nullptr;
+    if (status) {
+      const bool split = plan.splits > 1;  // the sum of the partials comes before bias and ReLU
+      const Conv3x3 conv{H, W, C, split ? nullptr : bias, split ? 0 : relu};
+      gemm_status_t st = f32tc_run(plan, a, sms, status, s, &conv);
+      if (st != GEMM_OK || !split || (!bias && !relu)) return st;
+      return kselect_bias_act(out, M, Cout, Cout, bias, relu, stream);
+    }
+  }
+  gemm_status_t st = kselect_im2col3x3(x, N, H, W, C, col, ld, stream);
+  if (st == GEMM_OK) st = gemm(h, 'N', 'T', M, Cout, K, 1.f, col, ld, weights, K, 0.f, out, Cout, 1, stream);
+  if (st == GEMM_OK && (bias || relu)) st = kselect_bias_act(out, M, Cout, Cout, bias, relu, stream);
+  return st;
+}
+
 gemm_status_t kselect_f32tc_selftest(int32_t bn, int32_t splits, char transA, char transB, int64_t M, int64_t N,
                                      int64_t K, float alpha, const float* A, int64_t lda, int64_t strideA,
                                      const float* B, int64_t ldb, int64_t strideB, float beta, float* C, int64_t ldc,
@@ -931,7 +982,7 @@ int32_t kselect_f32tc_choice(int32_t id, int64_t M, int64_t N, int64_t K, int64_
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return GEMM_ERR_CUDA;
   F32tcPlan plan;
-  if (noop || !f32tc_plan(id, a, dev, sm_count_of(dev), &plan)) return 0;
+  if (noop || !f32tc_plan(id, a, dev, sm_count_of(dev), 0.0, &plan)) return 0;
   *splits = plan.splits;
   return plan.bn;
 }

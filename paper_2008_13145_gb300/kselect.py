@@ -118,6 +118,7 @@ _sig("kselect_pca", i32, [i32, i32, vp, i32, i32, vp, vp, vp, vp, ctypes.POINTER
 _sig("kselect_pca_backproject", i32, [i32, i32, i32, vp, vp, vp, vp, vp])
 _sig("kselect_score", i32, [i32, i32, vp, i32, ctypes.POINTER(i32), vp, f32, ctypes.POINTER(f64), vp])
 _sig("kselect_im2col3x3", i32, [vp, i32, i32, i32, i32, vp, i64, vp])
+_sig("kselect_conv3x3", i32, [vp, vp, i32, i32, i32, i32, vp, i32, vp, i32, vp, i64, vp, vp])
 _sig("kselect_bias_act", i32, [vp, i64, i32, i64, vp, i32, vp])
 _sig("kselect_maxpool2x2", i32, [vp, i32, i32, i32, i32, vp, vp])
 _sig("kselect_im2col3x3_nchw", i32, [vp, i32, i32, i32, i32, vp, i64, vp])
@@ -492,6 +493,12 @@ def im2col3x3(x, N, H, W, C, out, ld, stream=None) -> None:
     check(_lib.kselect_im2col3x3(ptr(x), N, H, W, C, ptr(out), ld, stream_handle(stream)), "kselect_im2col3x3")
 
 
+def conv3x3(handle: Handle, x, N, H, W, C, weights, Cout, bias, relu, col, ld, out, stream=None) -> None:
+    """NHWC 3 x 3 convolution with bias and ReLU; `col` is scratch for the im2col rows (N H W x ld)."""
+    check(_lib.kselect_conv3x3(handle.value, ptr(x), N, H, W, C, ptr(weights), Cout, ptr(bias), int(relu), ptr(col),
+                               ld, ptr(out), stream_handle(stream)), "kselect_conv3x3")
+
+
 def bias_act(y, rows, cols, ld, bias, relu=True, stream=None) -> None:
     check(_lib.kselect_bias_act(ptr(y), rows, cols, ld, ptr(bias), int(relu), stream_handle(stream)), "kselect_bias_act")
 
@@ -760,7 +767,7 @@ def exported_symbols() -> list[str]:
             "gemm_config_params", "gemm_split_choose", "gemm_split_factor", "gemm_library_create", "gemm_library_destroy", "select_kernel", "gemm",
             "gemm_with_config", "gemm_host_pipeline", "gemm_strided_batched", "gemm_strided_batched_with_config", "gemm_host", "gemm_benchmark", "gemm_error_check", "kselect_fill_uniform",
             "gemm_benchmark_configs", "gemm_device_status", "kselect_wait_selftest", "kselect_f32tc_selftest", "kselect_f32tc_choice", "kselect_normalise", "kselect_kmeans", "kselect_score",
-            "kselect_im2col3x3", "kselect_bias_act", "kselect_maxpool2x2", "kselect_im2col3x3_nchw", "kselect_bias_act_nchw", "kselect_knn", "kselect_representatives", "kselect_top_n", "kselect_tree_regress", "kselect_tree_train", "kselect_tree_train_rf", "kselect_spectral_embedding", "kselect_cluster_geomean", "kselect_pca", "kselect_pca_backproject", "mlp_features", "mlp_forward", "mlp_loss_grad",
+            "kselect_im2col3x3", "kselect_conv3x3", "kselect_bias_act", "kselect_maxpool2x2", "kselect_im2col3x3_nchw", "kselect_bias_act_nchw", "kselect_knn", "kselect_representatives", "kselect_top_n", "kselect_tree_regress", "kselect_tree_train", "kselect_tree_train_rf", "kselect_spectral_embedding", "kselect_cluster_geomean", "kselect_pca", "kselect_pca_backproject", "mlp_features", "mlp_forward", "mlp_loss_grad",
             "mlp_adam_step", "mlp_loss_grad_noalloc", "mlp_train", "select_kernels_batched", "gemm_grouped_plan_create", "gemm_grouped_run",
             "gemm_grouped_plan_destroy", "gemm_grouped", "gemm_grouped_with_config", "gemm_grouped_reserve",
             "gemm_grouped_select", "kselect_selector_features", "kselect_best_labels", "mlp_targets"]

@@ -130,11 +130,8 @@ class VGG16:
                 continue
             if layer[0] == "conv":
                 _, h, ci, co = layer
-                M, K = n * h * h, 9 * ci
-                ldk = wl.round_up(K, 4)
-                ks.im2col3x3(cur, n, h, h, ci, self.col, ldk, stream)
-                ks.gemm(self.handle, "N", "T", M, co, K, 1.0, self.col, ldk, w[0], K, 0.0, out, co, 1, stream)
-                ks.bias_act(out, M, co, co, w[1], True, stream)
+                ks.conv3x3(self.handle, cur, n, h, h, ci, w[0], co, w[1], True, self.col, wl.round_up(9 * ci, 4), out,
+                           stream)
             elif layer[0] == "pool":
                 _, h, c = layer
                 ks.maxpool2x2(cur, n, h, h, c, out, stream)
