@@ -235,9 +235,13 @@ def run_ours(args, ws, rank, local):
     bufs = [tune.alloc_inputs(sh, ks.PREC_F32, 1000 + 7 * rank + i) for i, sh in enumerate(shapes)]
     flops = sum(sh.flops for sh in shapes)
     chosen = [ks.select_kernel(handle, sh.M, sh.N, sh.K, sh.batch) for sh in shapes]
-    # kernels per step: a split-K launch adds its reduction kernel
-    launches_per_step = sum(1 + (ks.split_factor(c, sh.M, sh.N, sh.K, sh.batch)[0] > 1)
-                            for c, sh in zip(chosen, shapes))
+    # What gemm() runs: the tensor cores at FP32 accuracy where it expects to gain
+    # by that ("f32tc"), else the selected config (the inputs' rows allow 16-byte access).
+    tc32 = [ks.f32tc_choice(c, sh.M, sh.N, sh.K, sh.batch, sh.transA) for c, sh in zip(chosen, shapes)]
+    ran = ["f32tc" if bn else c for c, (bn, _) in zip(chosen, tc32)]
+    # kernels per step: a split K adds its reduction kernel
+    launches_per_step = sum(1 + ((splits if bn else ks.split_factor(c, sh.M, sh.N, sh.K, sh.batch)[0]) > 1)
+                            for c, (bn, splits), sh in zip(chosen, tc32, shapes))
 
     def step(events=None, cfgs=None):
         for i, (sh, (A, B, C, lda, ldb, ldc)) in enumerate(zip(shapes, bufs)):
@@ -274,15 +278,15 @@ def run_ours(args, ws, rank, local):
     live = {"geomean": float(np.exp(np.mean(np.log(ratio)))), "mean": float(np.mean(ratio)),
             "source": "per-shape launch times this run, median of 3 passes each: exhaustive-best config vs "
                       "selected config"}
-    # Dominant kernel: the deployed config with the largest share of step time.
+    # Dominant kernel: the one with the largest share of step time.
     by_cfg = {}
-    for c, t, sh in zip(chosen, sel_ms, shapes):
+    for c, t, sh in zip(ran, sel_ms, shapes):
         a = by_cfg.setdefault(c, [0.0, 0, 0])
         a[0] += t
         a[1] += sh.flops
         a[2] += 1
     dom = max(by_cfg, key=lambda c: by_cfg[c][0])
-    dom_idx = [i for i, c in enumerate(chosen) if c == dom]
+    dom_idx = [i for i, c in enumerate(ran) if c == dom]
 
     # Timed region: K steps, dominant-kernel launches bracketed by events.
     dom_ev = [[(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in dom_idx]
@@ -395,14 +399,16 @@ def run_ours(args, ws, rank, local):
         "metric": METRIC, "value": value, "unit": "TFLOP/s", "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
-        "config": {"workload": WORKLOAD, "family": "FP32 SIMT", "deployed_kernels": len(dep["config_ids"]),
+        "config": {"workload": WORKLOAD,
+                   "family": "FP32 SIMT and split-K; FP32 accuracy on tensor cores (three BF16 parts, six products) "
+                             f"for the {sum(bool(bn) for bn, _ in tc32)} shapes where gemm() expects to gain",
+                   "deployed_kernels": len(dep["config_ids"]),
                    "selector": f"decision tree {dep['meta']['tree']}", "shapes_per_step": len(shapes),
                    "gflop_per_step": flops / 1e9, "l2": "inputs 7 GB per step, larger than L2",
                    "deployment": os.path.relpath(dep_path, ROOT)},
         "pct_of_exhaustive_optimum": {"live": live, "sweep_table_test_split": dep["meta"]["scores"]["tree"]},
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-                     "frac": achieved / FP32_PEAK_TFLOPS, "traffic": traffic, "kernel_config": dom,
-                     "kernel_params": ks.config_params(dom), "share_of_step": dom_share},
+        "roofline": {**fp32_roofline(achieved, dom == "f32tc"), "traffic": traffic, "kernel_config": dom,
+                     "kernel_params": None if dom == "f32tc" else ks.config_params(dom), "share_of_step": dom_share},
         "e2e": {"value": e2e, "unit": "TFLOP/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
         "selectors": selectors,
         "tc": tc,
@@ -567,11 +573,21 @@ def tc_large_shapes(ks, n: int = 8192, reps: int = 10, warmup: int = 3):
     return out
 
 
+def fp32_roofline(achieved: float, on_tensor_cores: bool) -> dict:
+    """Against the FP32 FMA peak, or a sixth of the measured BF16 rate where an FP32 product is six BF16 ones."""
+    peak = FP32_PEAK_TFLOPS
+    if on_tensor_cores:
+        path = os.path.join(ROOT, "MEASURED_PEAKS.json")
+        peak = (json.load(open(path))["bf16_tflops"] if os.path.exists(path) else 1900.0) / 6
+    return {"bound": "tensor" if on_tensor_cores else "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak}
+
+
 def fp32_large_shape(ks, n: int = 4096, reps: int = 10, warmup: int = 3):
-    """The FP32 SIMT family on one large product: n^3 NN through gemm() with the
-    FP32 deployment (its decision tree picks the kernel) and with each deployed
-    kernel directly, CUDA-event timed like tc_large_shapes (A, B and C together
-    exceed L2), against the FP32 FMA peak.  Beside it, as context only, the
+    """FP32 on one large product: n^3 NN through gemm() with the FP32 deployment
+    (which runs it on the tensor cores at FP32 accuracy where it expects to gain)
+    and with each deployed SIMT kernel directly, CUDA-event timed like
+    tc_large_shapes (A, B and C together exceed L2).  Beside it, as context only, the
     vendor library's FP32 GEMM on the same operands (torch.mm with TF32 off, i.e.
     cuBLAS computing in FP32 with FMA instructions), with the largest difference
     between its product and ours."""
@@ -616,8 +632,8 @@ def fp32_large_shape(ks, n: int = 4096, reps: int = 10, warmup: int = 3):
     best = max(per_cfg, key=per_cfg.get)
     return {"shape": f"{n}^3 NN", "timing": f"{warmup} warm-up + {reps} timed back-to-back launches",
             "value": tf, "unit": "TFLOP/s", "ms": ms, "config": ks.select_kernel(h, n, n, n, 1),
-            "roofline": {"bound": "alu", "achieved": tf, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-                         "frac": tf / FP32_PEAK_TFLOPS},
+            "f32tc_tile": ks.f32tc_choice(ks.select_kernel(h, n, n, n, 1), n, n, n)[0],
+            "roofline": fp32_roofline(tf, ks.f32tc_choice(ks.select_kernel(h, n, n, n, 1), n, n, n)[0] != 0),
             "deployed_configs": {str(c): v for c, v in per_cfg.items()}, "best_config": best,
             "best_value": per_cfg[best],
             "vendor_fp32_gemm_context": {"what": "torch.mm, TF32 off (cuBLAS FP32 GEMM)", "value": flops / (lib_ms * 1e9),

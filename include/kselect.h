@@ -619,9 +619,10 @@ gemm_status_t kselect_im2col3x3(const float* x_dev, int32_t N, int32_t H, int32_
  * neighbourhoods (kselect_im2col3x3) and the weights (Cout x 9 C, op(B) = B^T)
  * with the kernel the handle selects for those sizes, as the three calls
  * kselect_im2col3x3, gemm and kselect_bias_act give it (bias may be NULL, relu
- * 0).  Where C is a multiple of 32 and the tensor cores run the product at FP32
- * accuracy (see gemm), they read the image itself and add bias and ReLU as they
- * store; otherwise `col` (N*H*W rows of ld >= 9 C floats) receives the
+ * 0).  Where an FP32 kernel is selected, C is a multiple of 32 and the tensor
+ * cores run the product at FP32 accuracy (see gemm), they read the image itself
+ * and add bias and ReLU as they store, and so does a direct kernel for C <= 4;
+ * otherwise `col` (N*H*W rows of ld >= 9 C floats) receives the
  * neighbourhoods, and may not be NULL. */
 gemm_status_t kselect_conv3x3(gemm_handle_t handle, const float* x_dev, int32_t N, int32_t H, int32_t W, int32_t C,
                               const float* weights_dev, int32_t Cout, const float* bias_dev, int32_t relu,
@@ -687,7 +688,8 @@ gemm_status_t kselect_wait_selftest(int64_t limit_ns, int32_t* waited_out, void*
  * kselect_f32tc_selftest runs one, whatever gemm() would choose, with 128 x bn
  * tiles (bn 64 or 128) or 256 x 256 tiles on CTA pairs (bn 256) and K divided
  * into up to `splits` (1..16) ranges whose partial products a second kernel
- * sums; the other arguments are gemm_strided_batched's.  K = 0 is UNSUPPORTED.
+ * sums; the other arguments are gemm_strided_batched's.  K = 0 and K > 2^18 are
+ * UNSUPPORTED.
  * kselect_f32tc_choice returns the bn that a handle call uses instead of SIMT
  * config `config_id` (0: it runs the config), and the split factor, for these
  * sizes; `aligned` says whether every row allows 16-byte access.  Needs a GPU

@@ -108,6 +108,11 @@ struct Conv3x3 {
   int relu;
 };
 
+// 3 x 3 convolution of an image of few channels (vgg.cu).
+bool conv3x3_few_takes(int N, int H, int W, int C, int Cout, const float* bias, const float* out);
+cudaError_t conv3x3_few(const float* x, int N, int H, int W, int C, const float* w, int Cout, const float* bias,
+                        int relu, float* out, cudaStream_t s);
+
 using LaunchFn = cudaError_t (*)(const GemmArgs&, cudaStream_t);
 using OccFn = int (*)();  // resident CTAs per SM on the current device, 0 on error
 

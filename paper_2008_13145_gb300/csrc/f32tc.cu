@@ -231,8 +231,8 @@ struct Slice<R, kCols> {
 // outside.  A chunk then lies in one tap, and moving a tap on moves every row's
 // address by the same distance, so this is the K-contiguous slice with rows of
 // Ch, plus one bit per row and tap that says whether the tap is inside.  (Written
-// out by a separate pass, the neighbourhoods are nine times the image: 1.64 of
-// the 5.06 ms of VGG16 on 16 images.)
+// out by a separate pass, the neighbourhoods are nine times the image: VGG16 on
+// 16 images took 5.06 ms with that pass, and one for bias and ReLU, against 3.62.)
 template <int R>
 struct Slice<R, kConv> : Slice<R, kRows> {
   using Base = Slice<R, kRows>;

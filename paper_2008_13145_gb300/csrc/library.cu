@@ -400,6 +400,9 @@ constexpr double kF32tcSplitHostUs = 3.0;  // host work of a second launch and i
 // Below two K chunks the SIMT tiles, whose stores overlap other CTAs' loads,
 // stay ahead wherever they were measured to within the model's error.
 constexpr int kF32tcMinK = 64;
+// A tile that has to be computed again by FMAs takes up to 0.2 s at this K, well
+// inside the 2 s after which the kernel's other roles would give up waiting.
+constexpr int kF32tcMaxK = 1 << 18;
 constexpr int kF32tcChunk = 32;
 
 static double f32tc_cost(const F32tcCost& c, const GemmArgs& a, int64_t tiles, int64_t kc, int splits, int units) {
@@ -475,7 +478,7 @@ static bool f32tc_fastest(const GemmArgs& a, int sms, double limit_us, double li
 // Whether an FP32 request for which SIMT kernel `id` was selected runs on the
 // tensor cores, and how; other_us: what else the SIMT kernel would need first.
 static bool f32tc_plan(int id, const GemmArgs& a, int dev, int sms, double other_us, F32tcPlan* plan) {
-  if (a.K < kF32tcMinK || sms < 2) return false;
+  if (a.K < kF32tcMinK || a.K > kF32tcMaxK || sms < 2) return false;
   const double outputs = (double)a.M * (double)a.N * (double)a.batch;
   if (outputs > 1e12) return false;  // keeps the tile counts small
   if (2.0 * outputs * a.K < kF32tcMinFlops) return false;
@@ -917,23 +920,25 @@ gemm_status_t kselect_conv3x3(gemm_handle_t h, const float* x, int32_t N, int32_
   const int32_t id = select_kernel(h, M, Cout, K, 1);
   if (id < 0) return (gemm_status_t)id;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // FP32 classes, channels in whole K chunks, 16-byte rows: straight from the image.
-  const int fam = family_of(id);
+  // An FP32 kernel chosen, channels in whole K chunks or next to none: straight from
+  // the image.  (A split-BF16 choice keeps its three steps and with them its results.)
+  const bool fp32 = family_of(id) == GEMM_PREC_F32;
+  if (fp32 && conv3x3_few_takes(N, H, W, C, Cout, bias, out)) {
+    cudaError_t e = conv3x3_few(x, N, H, W, C, weights, Cout, bias, relu, out, s);
+    if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
+    return GEMM_OK;
+  }
   GemmArgs a;
   bool noop = false;
   int dev = 0;
-  if ((fam == GEMM_PREC_F32 || fam == GEMM_PREC_F32X3) && C % 32 == 0 && (uintptr_t)x % 16 == 0 &&
-      (uintptr_t)weights % 16 == 0 && cudaGetDevice(&dev) == cudaSuccess &&
+  if (fp32 && C % 32 == 0 && (uintptr_t)x % 16 == 0 && (uintptr_t)weights % 16 == 0 &&
+      cudaGetDevice(&dev) == cudaSuccess &&
       make_args('N', 'T', M, Cout, K, 1.f, x, K, weights, K, 0.f, out, Cout, 1, 4, &a, &noop) == GEMM_OK && !noop) {
     a.lda = C;  // of the image; its neighbourhoods are not stored
     const int sms = sm_count_of(dev);
     const double col_us = 2e6 * M * K * 4 / kSplitReduceBps;  // writing the neighbourhoods out and reading them back
     F32tcPlan plan;
-    // A split-BF16 choice is less exact, and needs the neighbourhoods split as well: it never stays ahead.
-    const bool use = fam == GEMM_PREC_F32 ? f32tc_plan(id, a, dev, sms, col_us, &plan)
-                                          : (double)M * Cout < 1e12 && 2.0 * M * Cout * K >= kF32tcMinFlops &&
-                                                sms >= 2 && f32tc_fastest(a, sms, INFINITY, INFINITY, &plan);
-    int* status = use ? status_word_for(s) : nullptr;
+    int* status = f32tc_plan(id, a, dev, sms, col_us, &plan) ? status_word_for(s) : nullptr;
     if (status) {
       const bool split = plan.splits > 1;  // the sum of the partials comes before bias and ReLU
       const Conv3x3 conv{H, W, C, split ? nullptr : bias, split ? 0 : relu};
@@ -958,7 +963,7 @@ gemm_status_t kselect_f32tc_selftest(int32_t bn, int32_t splits, char transA, ch
   gemm_status_t st = strided_args(0, transA, transB, M, N, K, alpha, A, lda, strideA, B, ldb, strideB, beta, C, ldc,
                                   strideC, batch, &a, &noop);
   if (st != GEMM_OK || noop) return st;
-  if (K == 0 || (double)M * (double)N * (double)batch > 1e12) return GEMM_ERR_UNSUPPORTED;
+  if (K == 0 || K > kF32tcMaxK || (double)M * (double)N * (double)batch > 1e12) return GEMM_ERR_UNSUPPORTED;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   int* status = e == cudaSuccess ? tc_status_word() : nullptr;

@@ -15,10 +15,12 @@ DEPLOY = os.path.join(os.path.dirname(os.path.abspath(vgg.__file__)), "deploy")
 
 # Images, height, width, channels, outputs: rows of one position, tiles across image ends,
 # every tile width (64, 128, 256 x 256), K split, the smallest channel count, sizes that
-# stay with the separate steps (few channels, little work).
+# stay with the separate steps (little work), and few channels.
 @pytest.mark.parametrize("n,H,W,C,Cout", [(1, 9, 1, 32, 700), (3, 37, 41, 64, 64), (2, 61, 50, 96, 130),
                                           (2, 70, 75, 128, 264), (1, 14, 14, 512, 512), (9, 33, 35, 32, 60),
-                                          (2, 12, 10, 3, 64), (1, 4, 4, 32, 8)])
+                                          (2, 12, 10, 3, 64), (1, 4, 4, 32, 8),
+                                          (1, 200, 52, 3, 64), (3, 61, 60, 1, 16), (2, 80, 64, 4, 256),
+                                          (2, 99, 100, 2, 48)])
 @pytest.mark.parametrize("deploy", ["f32.json", "f32mix.json"])
 def test_against_separate_steps(lib, n, H, W, C, Cout, deploy):
     import torch
