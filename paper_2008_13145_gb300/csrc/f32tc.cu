@@ -23,7 +23,11 @@
 // converting -- the third remainder then has bits below BF16's 16 -- and an
 // accumulator that overflowed is seen when it is read.  A tile that met either
 // is computed again by plain FP32 FMAs over K, so such inputs give what the
-// FP32 SIMT family gives.
+// FP32 SIMT family gives.  That is slow: one NaN takes 2048^3 from 85 us to
+// 11.6 ms (the SIMT kernel: 0.36 ms on any values), an infinity in every row of
+// 4096^3 from 621 us to 101 ms (SIMT: 2.5 ms).  Lanes with 2 or 4 rows by 4 columns
+// and 16-byte loads took 3.4 / 2.4 ms of the first, but the larger loop spills in
+// the whole kernel: ordinary 4096^3 went from 621 us to 669 / 813.
 //
 // One persistent CTA per SM, five warpgroups.
 //   8..15  : two groups that convert alternate chunks.  A thread loads its part

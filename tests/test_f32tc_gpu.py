@@ -73,7 +73,7 @@ def test_integers_exact_and_splits_repeatable(lib, torch, bn):
 
 
 @pytest.mark.parametrize("bn", [64, 128, 256])
-@pytest.mark.parametrize("kind", ["inf", "nan", "overflow", "tiny", "denormal", "zero"])
+@pytest.mark.parametrize("kind", ["inf", "nan", "overflow", "tiny", "denormal", "zero", "products"])
 def test_values_that_do_not_split(lib, torch, bn, kind):
     """Infinities, NaN, values that round past the largest BF16 and values whose low bits
     are below BF16's range give what the FP32 FMAs of the SIMT family give."""
@@ -90,6 +90,9 @@ def test_values_that_do_not_split(lib, torch, bn, kind):
         A[:, :, :sh.K] *= np.float32(2.0 ** -118)
     elif kind == "denormal":
         B[0, 9, :sh.K] *= np.float32(2.0 ** -140)
+    elif kind == "products":  # every factor splits, every product is denormal
+        A[:, :, :sh.K] *= np.float32(2.0 ** -70)
+        B[:, :, :sh.K] *= np.float32(2.0 ** -66)
     else:
         A[:, :, :sh.K] = 0
         B[0, 17, :sh.K] = -0.0
@@ -108,6 +111,22 @@ def test_values_that_do_not_split(lib, torch, bn, kind):
     ok = np.isfinite(want)
     # FMA chains of K terms, and results that are denormal themselves
     assert np.all(np.abs(got - ref)[ok] <= (sh.K + 2) * 2.0 ** -24 * den[ok] + sh.K * 2.0 ** -149)
+
+
+@pytest.mark.parametrize("trans", ["NN", "NT", "TN", "TT"])
+@pytest.mark.parametrize("bn,pad", [(64, 1), (128, 4), (256, 8), (256, 1)])
+def test_computed_again_in_every_layout(lib, torch, trans, bn, pad):
+    """Every tile by FMAs: each row of A holds a value whose low bits are below BF16's range."""
+    sh = wl.Shape(275, 261, 70, 2, trans[0], trans[1])
+    A, B, C0 = wl.gemm_inputs(sh, seed=11, ld_multiple=pad, beta_nonzero=True)
+    if trans[0] == "N":
+        A[:, :, 33] = np.float32(1.2345e-36)
+    else:
+        A[:, 33, :sh.M] = np.float32(1.2345e-36)
+    for splits in (1, 2):
+        got = run(lib, torch, bn, splits, sh, A, B, C0, 2.0, 0.5)
+        ref, den = og.gemm(sh.transA, sh.transB, sh.M, sh.N, sh.K, 2.0, A, B, 0.5, C0)
+        assert og.error_ratio(got, ref, den) <= (sh.K + 4) * 2.0 ** -24
 
 
 def test_shared_operand_strides(lib, torch):
