@@ -21,13 +21,14 @@
 // A split that is not exact (infinities, NaN, magnitudes whose low bits fall
 // below BF16's range, values that round past the largest BF16) is seen while
 // converting -- the third remainder then has bits below BF16's 16 -- and an
-// accumulator that overflowed is seen when it is read.  A tile that met either
-// is computed again by plain FP32 FMAs over K, so such inputs give what the
-// FP32 SIMT family gives.  That is slow: one NaN takes 2048^3 from 85 us to
-// 11.6 ms (the SIMT kernel: 0.36 ms on any values), an infinity in every row of
-// 4096^3 from 621 us to 101 ms (SIMT: 2.5 ms).  Lanes with 2 or 4 rows by 4 columns
-// and 16-byte loads took 3.4 / 2.4 ms of the first, but the larger loop spills in
-// the whole kernel: ordinary 4096^3 went from 621 us to 669 / 813.
+// accumulator that overflowed is seen when it is read.  A reading warp leaves
+// its part of such a tile unwritten and marks it; when all of the CTA's chunks
+// are summed, so that no role waits, the reading warps compute the marked parts
+// by plain FP32 FMAs over K (redo), so such inputs give what the FP32 SIMT family
+// gives.  One NaN takes 2048 x 2048 x 2048 from 85 to 563 us (SIMT kernel: 366, on
+// any values), an infinity in every row of 4096 x 4096 x 4096 from 595 to 4,410
+// (SIMT: 2,530): the parts of a tile stay with its SM.  (Computed where they were
+// met, by lanes with a row each: 11,640 and 101,000 us.)
 //
 // One persistent CTA per SM, five warpgroups.
 //   8..15  : two groups that convert alternate chunks.  A thread loads its part
@@ -45,6 +46,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -65,6 +67,7 @@ constexpr int kBK = 32;                       // K elements per chunk: one 64-by
 constexpr int kParts = 3;
 constexpr int kStoreBytes = 2048;             // staging of a reading warp's stores
 constexpr int kMarks = 16;                    // more than the chunks under way at once
+constexpr int kMaxItems = 1024;               // items of one CTA or pair: a byte each of `lost`
 
 // Stages: what fits in 164 KB, so that 92 KB are left as L1, where the FP32
 // loads under way land (with 28 KB left, the 256 x 256 tiles of 4096 x 4096 x
@@ -463,47 +466,175 @@ __device__ __forceinline__ void store_rows(const Args& p, const Item& it, int ro
   }
 }
 
-// `quads` groups of four columns of one row of an item by plain FP32 FMAs over
-// its K range, in K order.
-template <int AK, bool B_MN>
-__device__ __forceinline__ void redo_row(const Args& p, const Item& it, int row, int col, int quads) {
+// A block of an item, 32 rows row0 + 4 i by CW columns from col on, by plain FP32
+// FMAs over its K range, in K order; one warp, in its part of the emptied ring.  A
+// lane has 8 rows x 4 (CW 32) or 8 columns.  Eight K at a time go K-major into
+// shared memory by asynchronous copies of an element (any alignment, either
+// storage order; K-contiguous operands four rows of 32 bytes an instruction),
+// several steps ahead: what bounds a warp is their latency.  Pitches of 4 modulo 32
+// words keep the copies and the reads free of bank conflicts.
+template <int CW>
+struct Redo {
+  static constexpr int K = 8, APITCH = 36, BPITCH = CW + 4;
+  static constexpr int STEP = K * (APITCH + BPITCH);  // floats of one step
+  static constexpr int STEPS = CW == 32 ? 7 : 5;
+  static constexpr int FLOATS = STEPS * STEP;  // of one warp
+};
+
+// One element, or zero (`any` is then the address given).
+__device__ __forceinline__ void copy_async(uint32_t dst, const float* src, const float* any, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(in ? src : any), "r"(in ? 4 : 0)
+               : "memory");
+}
+
+template <int CW, int AK, bool B_MN>
+__device__ __forceinline__ void redo_block(const Args& p, const Item& it, int row0, int col, const float* buf,
+                                           int lane) {
+  using R = Redo<CW>;
   const GemmArgs& g = p.g;
-  if (row >= g.M) return;
-  const float* A = static_cast<const float*>(g.A) + (int64_t)it.b * g.strideA +
-                   (AK == kCols ? (int64_t)row : row * g.lda);
+  const float* A = static_cast<const float*>(g.A) + (int64_t)it.b * g.strideA;
   const float* B = static_cast<const float*>(g.B) + (int64_t)it.b * g.strideB;
-  float* crow = g.C + it.slab * g.strideC + (int64_t)row * g.ldc;
-  const int64_t as = AK == kCols ? g.lda : 1, bk = B_MN ? g.ldb : 1, bn = B_MN ? 1 : g.ldb;
-  int h = 0, w = 0;
+  const int four = lane >> 3, kk = lane & 7;  // K-contiguous: rows (columns) 4 e + four, K kk
+  uint32_t inside[AK == kConv ? 3 : 1];       // nine bits a row, three rows a word
   if constexpr (AK == kConv) {
-    const int hw = row % (p.H * p.W);
-    h = hw / p.W;
-    w = hw - h * p.W;
-  }
-#pragma unroll 1
-  for (int q = 0; q < quads; ++q) {
-    const int n = col + 4 * q;
-    if (n >= g.N) return;
-    const float* b[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) b[e] = B + min(n + e, g.N - 1) * bn;
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int k = it.kbeg; k < it.kend; ++k) {
-      float a;
-      if constexpr (AK == kConv) {
-        const int tap = k / p.Ch, dh = tap / 3 - 1, dw = tap % 3 - 1;
-        const bool in = (unsigned)(h + dh) < (unsigned)p.H && (unsigned)(w + dw) < (unsigned)p.W;
-        a = in ? __ldg(A + (int64_t)(dh * p.W + dw) * p.Ch + (k - tap * p.Ch)) : 0.f;
-      } else {
-        a = __ldg(A + k * as);
+    for (int i = 0; i < 3; ++i) inside[i] = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int m = row0 + 4 * (4 * e + four), hw = m % (p.H * p.W), h = hw / p.W, w = hw - h * p.W;
+      uint32_t in = 0;
+      if (m < g.M) {
+        const uint32_t cols = (w > 0 ? 1u : 0u) | 2u | (w + 1 < p.W ? 4u : 0u);
+        in = (h > 0 ? cols : 0u) | cols << 3 | (h + 1 < p.H ? cols << 6 : 0u);
+      }
+      inside[e / 3] |= in << (9 * (e % 3));
+    }
+  }
+  const uint32_t sbuf = smem_u32(buf);
+  // INNER: every element of the step exists, which spares the copies their tests.
+  auto copies = [&](int k0, uint32_t sa, uint32_t sb, auto inner) {
+    constexpr bool INNER = decltype(inner)::value;
+    const int left = it.kend - k0;
+    if constexpr (AK == kCols) {
+      const float* a = A + k0 * g.lda + row0 + 4 * lane;
+      const bool row = row0 + 4 * lane < g.M;
+#pragma unroll
+      for (int e = 0; e < R::K; ++e, a += g.lda)
+        copy_async(sa + 4 * (e * R::APITCH + lane), a, A, INNER || (row && e < left));
+    } else if constexpr (AK == kConv) {
+      const int tap = k0 / p.Ch;  // a step is in one tap
+      const float* a =
+          A + ((int64_t)row0 + 4 * four + (tap / 3 - 1) * p.W + (tap % 3 - 1)) * p.Ch + (k0 - tap * p.Ch) + kk;
+#pragma unroll
+      for (int e = 0; e < 8; ++e, a += 16 * p.Ch)
+        copy_async(sa + 4 * (kk * R::APITCH + 4 * e + four), a, A, (inside[e / 3] >> (9 * (e % 3) + tap)) & 1);
+    } else {
+      const float* a = A + (int64_t)(row0 + 4 * four) * g.lda + k0 + kk;
+#pragma unroll
+      for (int e = 0; e < 8; ++e, a += 16 * g.lda)
+        copy_async(sa + 4 * (kk * R::APITCH + 4 * e + four), a, A,
+                   INNER || (row0 + 4 * (4 * e + four) < g.M && kk < left));
+    }
+    if constexpr (B_MN) {
+      const float* b = B + k0 * g.ldb + col + lane;
+#pragma unroll
+      for (int e = 0; e < R::K; ++e, b += g.ldb)
+#pragma unroll
+        for (int c = 0; c < CW; c += 32)
+          copy_async(sb + 4 * (e * R::BPITCH + c + lane), b + c, B, INNER || (col + c + lane < g.N && e < left));
+    } else {
+      const float* b = B + (int64_t)(col + four) * g.ldb + k0 + kk;
+#pragma unroll
+      for (int e = 0; e < CW / 4; ++e, b += 4 * g.ldb)
+        copy_async(sb + 4 * (kk * R::BPITCH + 4 * e + four), b, B,
+                   INNER || (col + 4 * e + four < g.N && kk < left));
+    }
+  };
+  // (Not with A^T: the pair kernel of A^T B then takes 720 us at 4096 x 4096 x 4096
+  // on values that all split, 581 without.)
+  const bool whole = AK != kCols && row0 + 4 * 31 < g.M && col + CW <= g.N;
+  auto load = [&](int step) {
+    const int k0 = it.kbeg + step * R::K;
+    const uint32_t sa = sbuf + 4 * (step % R::STEPS * R::STEP), sb = sa + 4 * R::K * R::APITCH;
+    if (whole && k0 + R::K <= it.kend) copies(k0, sa, sb, std::true_type());
+    else if (k0 < it.kend) copies(k0, sa, sb, std::false_type());
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int r0 = 8 * (lane >> 3), c0 = 4 * (lane & 7), steps = (it.kend - it.kbeg + R::K - 1) / R::K;
+  float v[8][CW / 8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < CW / 8; ++j) v[i][j] = 0.f;
+  __syncwarp();  // the block before is summed
+#pragma unroll 1
+  for (int s = 0; s < R::STEPS - 1; ++s) load(s);
+#pragma unroll 1
+  for (int s = 0; s < steps; ++s) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(R::STEPS - 2) : "memory");
+    __syncwarp();
+    load(s + R::STEPS - 1);
+    const float* sa = buf + s % R::STEPS * R::STEP;
+    const float* sb = sa + R::K * R::APITCH;
+#pragma unroll
+    for (int k = 0; k < R::K; ++k) {  // past the range both operands are zero
+      float a[8], b[CW / 8];
+#pragma unroll
+      for (int i = 0; i < 8; i += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(sa + k * R::APITCH + r0 + i);
+        a[i] = t.x; a[i + 1] = t.y; a[i + 2] = t.z; a[i + 3] = t.w;
       }
 #pragma unroll
-      for (int e = 0; e < 4; ++e) v[e] = fmaf(a, __ldg(b[e] + k * bk), v[e]);
+      for (int j = 0; j < CW / 8; j += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(sb + k * R::BPITCH + 8 * j + c0);
+        b[j] = t.x; b[j + 1] = t.y; b[j + 2] = t.z; b[j + 3] = t.w;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < CW / 8; ++j) v[i][j] = fmaf(a[i], b[j], v[i][j]);
     }
-    store4<AK == kConv>(p, crow + n, n, g.N - n, v);
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int row = row0 + 4 * (r0 + i);
+    float* crow = g.C + it.slab * g.strideC + (int64_t)row * g.ldc;
+#pragma unroll
+    for (int j = 0; j < CW / 8; j += 4) {
+      const int n = col + 8 * j + c0;
+      const float o[4] = {v[i][j], v[i][j + 1], v[i][j + 2], v[i][j + 3]};
+      if (row < g.M && n < g.N) store4<AK == kConv>(p, crow + n, n, g.N - n, o);
+    }
   }
 }
+
+// What the reading warps left unwritten: byte o of `lost` has a bit for each
+// warp's part of the CTA's item first + o * step.  The parts, or halves of a pair's,
+// go round the reading warps.
+template <int BN, int BM, int G, int AK, bool B_MN>
+__device__ __forceinline__ void redo(const Args& p, const uint32_t* lost, int first, int step, int m_off,
+                                     const float* ring, int warp, int lane) {
+  constexpr int CW = G == 8 ? 32 : 64;
+  int turn = 0;
+#pragma unroll 1
+  for (int o = 0; first + (int64_t)o * step < p.items; ++o) {
+    uint32_t bits = (lost[o >> 2] >> (8 * (o & 3))) & 255u;
+    if (!bits) continue;
+    const Item it = item_of<BN, BM>(p, first + o * step);
+#pragma unroll 1
+    for (; bits; bits &= bits - 1) {
+      const int w = __ffs(bits) - 1, row0 = it.m0 + m_off + (w & 3), col = it.n0 + 4 * G * (w >> 2);
+#pragma unroll 1
+      for (int c = col; c < min(col + 4 * G, p.g.N); c += CW)
+        if (turn++ % kReaders == warp)
+          redo_block<CW, AK, B_MN>(p, it, row0, c, ring + warp * Redo<CW>::FLOATS, lane);
+    }
+  }
+}
+
+// The reading warps have all left their loops.
+__device__ __forceinline__ void readers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kReaders) : "memory"); }
 
 template <int BN, int AK, bool B_MN>
 __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constant__ Args p) {
@@ -512,6 +643,8 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t full[C::STAGES], empty[C::STAGES], accf[2], acce[2];
   __shared__ int inexact[kMarks];  // chunk i left its mark i + 1 in slot i % kMarks when a split lost bits
+  __shared__ uint32_t lost_sh[kMaxItems / 4];  // see redo
+  __shared__ int any_lost;
   __shared__ uint32_t tmem_sh;
   const uint32_t smem = (smem_u32(smem_raw) + 1023) & ~1023u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -528,6 +661,8 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
     fence_barrier_init();
   }
   if (threadIdx.x < kMarks) inexact[threadIdx.x] = 0;
+  if (threadIdx.x < kMaxItems / 4) lost_sh[threadIdx.x] = 0;
+  if (threadIdx.x == 0) any_lost = 0;
   if (warp == kIssuer) tmem_alloc<C::TMEM>(&tmem_sh);
   tc_fence_before();
   __syncthreads();
@@ -628,7 +763,7 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
     if constexpr (C::REGS_READ > kRegsLaunch) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::REGS_READ));
     float acc[4][G];
     int item = blockIdx.x, at = 0, n = 0;  // the item being summed, chunks of it added, its chunks
-    bool lost = false;
+    bool lost = false, whole = true;
     const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * G);
     const uint32_t stage = smem + C::STAGES * C::STAGE + warp * kStoreBytes;
     for (int c = 0; c < total; ++c) {
@@ -640,8 +775,8 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
 #pragma unroll
           for (int q = 0; q < G; ++q) acc[j][q] = 0.f;
       }
-      if (!warp_wait(&accf[c & 1], (c >> 1) & 1, p.status, kStatusTimeoutAcc)) break;
-      __syncwarp();  // lanes without a row of C, or with one to compute again, may have been elsewhere
+      if (!(whole = warp_wait(&accf[c & 1], (c >> 1) & 1, p.status, kStatusTimeoutAcc))) break;
+      __syncwarp();  // lanes without a row of C may have been elsewhere
       tc_fence_after();
       lost |= *(volatile int*)&inexact[c % kMarks] == c + 1;
 #pragma unroll
@@ -663,20 +798,36 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
       item += gridDim.x;
       const int row0 = it.m0 + (warp & 3), col = it.n0 + 4 * G * (warp >> 2);
       if (row0 >= p.g.M || col >= p.g.N) continue;
-      // A split that lost bits or an accumulator that overflowed: plain FP32 FMAs.
+      // A split that lost bits or an accumulator that overflowed: left to redo().
 #pragma unroll
       for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int q = 0; q < G; ++q) lost |= !(fabsf(acc[j][q]) <= 3.402823466e38f);
-      if (__any_sync(0xffffffffu, lost)) redo_row<AK, B_MN>(p, it, row0 + 4 * lane, col, G);
-      else store_rows<G, AK == kConv>(p, it, row0, col, acc, stage, lane);
+      if (!__any_sync(0xffffffffu, lost)) {
+        store_rows<G, AK == kConv>(p, it, row0, col, acc, stage, lane);
+      } else if (lane == 0) {
+        const int o = (item - (int)blockIdx.x) / (int)gridDim.x - 1;
+        atomicOr(&lost_sh[o >> 2], 1u << (8 * (o & 3) + warp));
+        any_lost = 1;
+      }
     }
+    readers_sync();
+    if (whole && *(volatile int*)&any_lost)
+      redo<BN, kBM, G, AK, B_MN>(p, lost_sh, blockIdx.x, gridDim.x, 0,
+                                 reinterpret_cast<float*>(smem_raw + (smem - smem_u32(smem_raw))), warp, lane);
   }
   __syncthreads();
   if (warp == kIssuer) {
     tc_fence_after();
     tmem_dealloc<C::TMEM>(tmem);
   }
+}
+
+// CTAs or pairs of a launch: as many as are resident at once, and whole multiples
+// of that where each would have more items than it can mark.
+int units_for(int items, int resident) {
+  const int64_t most = (int64_t)resident * kMaxItems;
+  return (int)std::min<int64_t>(items, resident * ((items + most - 1) / most));
 }
 
 template <int BN, int AK, bool B_MN>
@@ -695,7 +846,7 @@ cudaError_t launch(const Args& a, int sms, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     __atomic_fetch_or(&done_mask, bit, __ATOMIC_ACQ_REL);
   }
-  return launch_pdl(kern, dim3((unsigned)std::min(a.items, sms)), dim3(kThreads), Cfg<BN>::SMEM, s, nullptr, 0, a);
+  return launch_pdl(kern, dim3((unsigned)units_for(a.items, sms)), dim3(kThreads), Cfg<BN>::SMEM, s, nullptr, 0, a);
 }
 
 template <int BN>
@@ -802,6 +953,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t full[Pair::STAGES], empty[Pair::STAGES], accf[2], acce[2];
   __shared__ int inexact[kMarks];
+  __shared__ uint32_t lost_sh[kMaxItems / 4];
+  __shared__ int any_lost;
   __shared__ uint32_t tmem_sh;
   const uint32_t smem = (smem_u32(smem_raw) + 1023) & ~1023u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -820,6 +973,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     fence_barrier_init();
   }
   if (threadIdx.x < kMarks) inexact[threadIdx.x] = 0;
+  if (threadIdx.x < kMaxItems / 4) lost_sh[threadIdx.x] = 0;
+  if (threadIdx.x == 0) any_lost = 0;
   if (warp == kIssuer) tmem_alloc_pair<Pair::TMEM>(&tmem_sh);
   tc_fence_before();
   __syncthreads();
@@ -861,7 +1016,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPairRegsRead));
     float acc[4][G];
     int item = unit, at = 0, n = 0;
-    bool lost = false;
+    bool lost = false, whole = true;
     const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 128);
     const uint32_t stage = smem + Pair::STAGES * Pair::STAGE + warp * kStoreBytes;
     for (int c = 0; c < total; ++c) {
@@ -873,7 +1028,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int q = 0; q < G; ++q) acc[j][q] = 0.f;
       }
-      if (!warp_wait(&accf[c & 1], (c >> 1) & 1, p.status, kStatusTimeoutAcc)) break;
+      if (!(whole = warp_wait(&accf[c & 1], (c >> 1) & 1, p.status, kStatusTimeoutAcc))) break;
       __syncwarp();
       tc_fence_after();
       lost |= *(volatile int*)&inexact[c % kMarks] == c + 1;
@@ -896,14 +1051,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       item += units;
       const int row0 = it.m0 + 128 * (int)rank + (warp & 3), col = it.n0 + 128 * (warp >> 2);
       if (row0 >= p.g.M || col >= p.g.N) continue;
-      // A split that lost bits or an accumulator that overflowed: plain FP32 FMAs.
+      // A split that lost bits or an accumulator that overflowed: left to redo().
 #pragma unroll
       for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int q = 0; q < G; ++q) lost |= !(fabsf(acc[j][q]) <= 3.402823466e38f);
-      if (__any_sync(0xffffffffu, lost)) redo_row<AK, B_MN>(p, it, row0 + 4 * lane, col, G);
-      else store_rows<G, AK == kConv>(p, it, row0, col, acc, stage, lane);
+      if (!__any_sync(0xffffffffu, lost)) {
+        store_rows<G, AK == kConv>(p, it, row0, col, acc, stage, lane);
+      } else if (lane == 0) {
+        const int o = (item - unit) / units - 1;
+        atomicOr(&lost_sh[o >> 2], 1u << (8 * (o & 3) + warp));
+        any_lost = 1;
+      }
     }
+    readers_sync();
+    if (whole && *(volatile int*)&any_lost)
+      redo<Pair::BN, Pair::BM, G, AK, B_MN>(p, lost_sh, unit, units, 128 * (int)rank,
+                                            reinterpret_cast<float*>(smem_raw + (smem - smem_u32(smem_raw))), warp,
+                                            lane);
   }
   __syncthreads();
   cluster_sync();  // neither CTA leaves while the other's MMAs or arrivals may reach it
@@ -929,7 +1094,7 @@ cudaError_t launch_pair(const Args& a, int sms, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     __atomic_fetch_or(&done_mask, bit, __ATOMIC_ACQ_REL);
   }
-  const int pairs = std::min(a.items, sms / 2);
+  const int pairs = units_for(a.items, sms / 2);
   return launch_pdl(kern, dim3((unsigned)(2 * pairs)), dim3(kThreads), Pair::SMEM, s, nullptr, 0, a);
 }
 

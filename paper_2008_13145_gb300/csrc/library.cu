@@ -400,8 +400,8 @@ constexpr double kF32tcSplitHostUs = 3.0;  // host work of a second launch and i
 // Below two K chunks the SIMT tiles, whose stores overlap other CTAs' loads,
 // stay ahead wherever they were measured to within the model's error.
 constexpr int kF32tcMinK = 64;
-// A tile that has to be computed again by FMAs takes up to 0.2 s at this K, well
-// inside the 2 s after which the kernel's other roles would give up waiting.
+// The models were fitted to K up to 4096; the kernels are tested up to this K, on
+// values that split and on values that do not.
 constexpr int kF32tcMaxK = 1 << 18;
 constexpr int kF32tcChunk = 32;
 
