@@ -65,10 +65,11 @@ int32_t gemm_last_cuda_error(void);
 
 /* Debug-build hooks (no paper counterpart).  The library built with
  * KS_DEBUG_BOUNDS (libkselect_debug.so, a subset of the FP32 configs) checks
- * every global access of its FP32 kernels and of the split-K reduction
- * against the bytes each operand may span from its base -- (batch - 1)
- * strides + (rows - 1) leading dimensions + the row length -- and counts and
- * skips any access outside.  kselect_debug_bounds_errors reads the count
+ * every global access to A, B and C of its FP32 GEMM kernels (SIMT, and the
+ * tensor cores at FP32 accuracy) and of the split-K reduction against the
+ * bytes each operand may span from its base -- (batch - 1) strides + (rows - 1)
+ * leading dimensions + the row length; of a convolution's image its size --
+ * and counts and skips any access outside.  kselect_debug_bounds_errors reads the count
  * (synchronising the device; clear != 0 resets it); kselect_debug_shrink_extents
  * declares the operand extents smaller by the given bytes on later calls (a
  * test of the checker itself, which then flags accesses that are in fact

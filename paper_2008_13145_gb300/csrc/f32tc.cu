@@ -137,6 +137,14 @@ __device__ __forceinline__ uint32_t swz64(int row, int byte) {  // 64-byte rows,
 __device__ __forceinline__ void sts64(uint32_t addr, uint32_t x, uint32_t y) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(x), "r"(y) : "memory");
 }
+// Elements of operand `op` (0 = A, 1 = B); zero where the debug build finds them out of bounds.
+__device__ __forceinline__ float load1(const GemmArgs& g, int op, const float* p) {
+  return ks_in_bounds(g, op, p, 4) ? __ldg(p) : 0.f;
+}
+__device__ __forceinline__ float4 load4(const GemmArgs& g, int op, const float* p) {
+  return ks_in_bounds(g, op, p, 16) ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 // One operand's slice of R rows (M of A, N of B) x 32 K as this thread loads and
 // stores it.
 template <int R, int KIND>
@@ -164,16 +172,17 @@ struct Slice<R, kRows> {
     step = 16 * ld;
   }
   __device__ __forceinline__ void advance() { ptr += kBK; }
-  __device__ __forceinline__ void load(int t, float (&v)[N], bool fast, bool vec, int kleft) const {
+  __device__ __forceinline__ void load(const GemmArgs& g, int op, int t, float (&v)[N], bool fast, bool vec,
+                                       int kleft) const {
     const float* p = ptr + t * step;
     const int left = fast ? kBK : kleft - 4 * kq;
     const bool in = fast || 16 * t < lim;
     if (fast || (in && vec && left >= 4)) {
-      const float4 x = __ldg(reinterpret_cast<const float4*>(p));
+      const float4 x = load4(g, op, p);
       v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
     } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) v[e] = (in && e < left) ? __ldg(p + e) : 0.f;
+      for (int e = 0; e < 4; ++e) v[e] = (in && e < left) ? load1(g, op, p + e) : 0.f;
     }
   }
   __device__ __forceinline__ void store(int t, const float (&v)[N], uint32_t base, uint32_t& rem) const {
@@ -206,17 +215,18 @@ struct Slice<R, kCols> {
     ptr = base + (int64_t)(k0 + k) * ld + r0 + row;
   }
   __device__ __forceinline__ void advance() { ptr += kBK * ld; }
-  __device__ __forceinline__ void load(int t, float (&v)[N], bool fast, bool vec, int kleft) const {
+  __device__ __forceinline__ void load(const GemmArgs& g, int op, int t, float (&v)[N], bool fast, bool vec,
+                                       int kleft) const {
     const float* p = ptr + 16 * t * ld;
 #pragma unroll
     for (int e = 0; e < 4; ++e, p += ld) {
       const bool in = fast || k + 16 * t + e < kleft;
       if (fast || (in && vec && lim >= 4)) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(p));
+        const float4 x = load4(g, op, p);
         v[4 * e] = x.x; v[4 * e + 1] = x.y; v[4 * e + 2] = x.z; v[4 * e + 3] = x.w;
       } else {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v[4 * e + j] = (in && j < lim) ? __ldg(p + j) : 0.f;
+        for (int j = 0; j < 4; ++j) v[4 * e + j] = (in && j < lim) ? load1(g, op, p + j) : 0.f;
       }
     }
   }
@@ -277,10 +287,10 @@ struct Slice<R, kConv> : Slice<R, kRows> {
       if (++tap % 3 == 0) this->ptr += down;
     }
   }
-  __device__ __forceinline__ void load(int t, float (&v)[N], bool, bool, int) const {
+  __device__ __forceinline__ void load(const GemmArgs& g, int op, int t, float (&v)[N], bool, bool, int) const {
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
     if ((inside[t / 3] >> (9 * (t % 3) + tap)) & 1)
-      x = __ldg(reinterpret_cast<const float4*>(this->ptr + t * this->step));
+      x = load4(g, op, this->ptr + t * this->step);
     v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
   }
 };
@@ -372,6 +382,7 @@ template <bool ACT>
 __device__ __forceinline__ void store4(const Args& p, float* dst, int n, int left, const float (&v)[4]) {
   const GemmArgs& g = p.g;
   float o[4] = {g.alpha * v[0], g.alpha * v[1], g.alpha * v[2], g.alpha * v[3]};
+  if (!ks_in_bounds(g, 2, dst, 4 * min(left, 4))) return;
   if (g.vecC && left >= 4) {
     if (g.beta != 0.f) {
       const float4 c = *reinterpret_cast<const float4*>(dst);
@@ -408,6 +419,7 @@ __device__ __forceinline__ void store_rows(const Args& p, const Item& it, int ro
 #pragma unroll
       for (int e = 0; e < 8; ++e) o[e] = alpha * acc[e & 3][q + (e >> 2)];
       float* dst = crow + 4 * q;
+      if (!ks_in_bounds(p.g, 2, dst, 32)) continue;
       if (beta != 0.f) {
         const float4 c0 = *reinterpret_cast<const float4*>(dst), c1 = *reinterpret_cast<const float4*>(dst + 4);
         o[0] = fmaf(beta, c0.x, o[0]); o[1] = fmaf(beta, c0.y, o[1]);
@@ -458,6 +470,7 @@ __device__ __forceinline__ void store_rows(const Args& p, const Item& it, int ro
                      : "memory");
         if (row < p.g.M && c < left) {
           float* dst = base + (int64_t)row * p.g.ldc + 16 * blk + c;
+          if (!ks_in_bounds(p.g, 2, dst, 4)) continue;
           o *= alpha;
           *dst = act<ACT>(p, col + 16 * blk + c, beta != 0.f ? fmaf(beta, *dst, o) : o);
         }
@@ -481,8 +494,10 @@ struct Redo {
   static constexpr int FLOATS = STEPS * STEP;  // of one warp
 };
 
-// One element, or zero (`any` is then the address given).
-__device__ __forceinline__ void copy_async(uint32_t dst, const float* src, const float* any, bool in) {
+// One element of operand `op`, or zero (its base `any` is then the address given).
+__device__ __forceinline__ void copy_async(const GemmArgs& g, int op, uint32_t dst, const float* src,
+                                           const float* any, bool in) {
+  in = in && ks_in_bounds(g, op, src, 4);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(in ? src : any), "r"(in ? 4 : 0)
                : "memory");
 }
@@ -520,19 +535,19 @@ __device__ __forceinline__ void redo_block(const Args& p, const Item& it, int ro
       const bool row = row0 + 4 * lane < g.M;
 #pragma unroll
       for (int e = 0; e < R::K; ++e, a += g.lda)
-        copy_async(sa + 4 * (e * R::APITCH + lane), a, A, INNER || (row && e < left));
+        copy_async(g, 0, sa + 4 * (e * R::APITCH + lane), a, A, INNER || (row && e < left));
     } else if constexpr (AK == kConv) {
       const int tap = k0 / p.Ch;  // a step is in one tap
       const float* a =
           A + ((int64_t)row0 + 4 * four + (tap / 3 - 1) * p.W + (tap % 3 - 1)) * p.Ch + (k0 - tap * p.Ch) + kk;
 #pragma unroll
       for (int e = 0; e < 8; ++e, a += 16 * p.Ch)
-        copy_async(sa + 4 * (kk * R::APITCH + 4 * e + four), a, A, (inside[e / 3] >> (9 * (e % 3) + tap)) & 1);
+        copy_async(g, 0, sa + 4 * (kk * R::APITCH + 4 * e + four), a, A, (inside[e / 3] >> (9 * (e % 3) + tap)) & 1);
     } else {
       const float* a = A + (int64_t)(row0 + 4 * four) * g.lda + k0 + kk;
 #pragma unroll
       for (int e = 0; e < 8; ++e, a += 16 * g.lda)
-        copy_async(sa + 4 * (kk * R::APITCH + 4 * e + four), a, A,
+        copy_async(g, 0, sa + 4 * (kk * R::APITCH + 4 * e + four), a, A,
                    INNER || (row0 + 4 * (4 * e + four) < g.M && kk < left));
     }
     if constexpr (B_MN) {
@@ -541,12 +556,12 @@ __device__ __forceinline__ void redo_block(const Args& p, const Item& it, int ro
       for (int e = 0; e < R::K; ++e, b += g.ldb)
 #pragma unroll
         for (int c = 0; c < CW; c += 32)
-          copy_async(sb + 4 * (e * R::BPITCH + c + lane), b + c, B, INNER || (col + c + lane < g.N && e < left));
+          copy_async(g, 1, sb + 4 * (e * R::BPITCH + c + lane), b + c, B, INNER || (col + c + lane < g.N && e < left));
     } else {
       const float* b = B + (int64_t)(col + four) * g.ldb + k0 + kk;
 #pragma unroll
       for (int e = 0; e < CW / 4; ++e, b += 4 * g.ldb)
-        copy_async(sb + 4 * (kk * R::BPITCH + 4 * e + four), b, B,
+        copy_async(g, 1, sb + 4 * (kk * R::BPITCH + 4 * e + four), b, B,
                    INNER || (col + 4 * e + four < g.N && kk < left));
     }
   };
@@ -720,9 +735,9 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
       for (int s = 0; s < group; ++s) skip();
       const bool wa = fa && left >= kBK, wb = fb && left >= kBK;
 #pragma unroll
-      for (int t = 0; t < SA::PARTS; ++t) sa.load(t, va[t], wa, p.g.vecA, left);
+      for (int t = 0; t < SA::PARTS; ++t) sa.load(p.g, 0, t, va[t], wa, p.g.vecA, left);
 #pragma unroll
-      for (int t = 0; t < SB::PARTS; ++t) sb.load(t, vb[t], wb, p.g.vecB, left);
+      for (int t = 0; t < SB::PARTS; ++t) sb.load(p.g, 1, t, vb[t], wb, p.g.vecB, left);
     }
     for (int i = group; i < total; i += kGroups) {
       const int stage = i % C::STAGES;
@@ -736,11 +751,11 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
 #pragma unroll
         for (int t = 0; t < SA::PARTS; ++t) sa.store(t, va[t], a0, rem);
 #pragma unroll
-        for (int t = 0; t < SA::PARTS; ++t) sa.load(t, va[t], true, true, left);
+        for (int t = 0; t < SA::PARTS; ++t) sa.load(p.g, 0, t, va[t], true, true, left);
 #pragma unroll
         for (int t = 0; t < SB::PARTS; ++t) sb.store(t, vb[t], b0, rem);
 #pragma unroll
-        for (int t = 0; t < SB::PARTS; ++t) sb.load(t, vb[t], true, true, left);
+        for (int t = 0; t < SB::PARTS; ++t) sb.load(p.g, 1, t, vb[t], true, true, left);
       } else {
 #pragma unroll
         for (int t = 0; t < SA::PARTS; ++t) sa.store(t, va[t], a0, rem);
@@ -748,9 +763,9 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
         for (int t = 0; t < SB::PARTS; ++t) sb.store(t, vb[t], b0, rem);
         if (more) {
 #pragma unroll
-          for (int t = 0; t < SA::PARTS; ++t) sa.load(t, va[t], false, p.g.vecA, left);
+          for (int t = 0; t < SA::PARTS; ++t) sa.load(p.g, 0, t, va[t], false, p.g.vecA, left);
 #pragma unroll
-          for (int t = 0; t < SB::PARTS; ++t) sb.load(t, vb[t], false, p.g.vecB, left);
+          for (int t = 0; t < SB::PARTS; ++t) sb.load(p.g, 1, t, vb[t], false, p.g.vecB, left);
         }
       }
       if (rem & 0xffffu) inexact[i % kMarks] = i + 1;
@@ -904,7 +919,7 @@ __device__ __forceinline__ void convert_pair(const Args& p, int total, bool is_a
     skip();
     const bool whole = inner && left >= kBK;
 #pragma unroll
-    for (int t = 0; t < S::PARTS; ++t) sl.load(t, v[t], whole, vec, left);
+    for (int t = 0; t < S::PARTS; ++t) sl.load(p.g, is_a ? 0 : 1, t, v[t], whole, vec, left);
   }
   for (int i = 0; i < total; ++i) {
     const int stage = i % Pair::STAGES;
@@ -924,14 +939,14 @@ __device__ __forceinline__ void convert_pair(const Args& p, int total, bool is_a
 #pragma unroll
         for (int t = h; t < h + H; ++t) sl.store(t, v[t], at, rem);
 #pragma unroll
-        for (int t = h; t < h + H; ++t) sl.load(t, v[t], true, true, left);
+        for (int t = h; t < h + H; ++t) sl.load(p.g, is_a ? 0 : 1, t, v[t], true, true, left);
       }
     } else {
 #pragma unroll
       for (int t = 0; t < S::PARTS; ++t) sl.store(t, v[t], at, rem);
       if (more) {
 #pragma unroll
-        for (int t = 0; t < S::PARTS; ++t) sl.load(t, v[t], false, vec, left);
+        for (int t = 0; t < S::PARTS; ++t) sl.load(p.g, is_a ? 0 : 1, t, v[t], false, vec, left);
       }
     }
     if (rem & 0xffffu) {  // B's columns are in both CTAs' rows of C

@@ -498,8 +498,9 @@ static gemm_status_t f32tc_run(const F32tcPlan& plan, const GemmArgs& a, int sms
     return GEMM_OK;
   }
   const int64_t ldw = ((int64_t)a.N + 7) / 8 * 8;
+  const size_t bytes = (size_t)splits * a.batch * a.M * ldw * sizeof(float);
   void* w = nullptr;
-  e = scratch_alloc(&w, (size_t)splits * a.batch * a.M * ldw * sizeof(float), s);
+  e = scratch_alloc(&w, bytes, s);
   if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
   GemmArgs p = a;
   p.alpha = 1.f;
@@ -508,12 +509,21 @@ static gemm_status_t f32tc_run(const F32tcPlan& plan, const GemmArgs& a, int sms
   p.ldc = ldw;
   p.strideC = ldw * a.M;
   p.vecC = 1;
+#ifdef KS_DEBUG_BOUNDS
+  p.lo[2] = static_cast<const char*>(w);  // as in launch_split
+  p.ext[2] = (int64_t)bytes;
+  GemmArgs chk = a;
+  chk.lo[0] = static_cast<const char*>(w);
+  chk.ext[0] = (int64_t)bytes;
+#else
+  const GemmArgs& chk = a;
+#endif
   e = f32tc_launch(bn, p, splits, kchunk, sms, status, s, conv);
   if (e == cudaSuccess) {
     const int64_t total = (int64_t)a.batch * a.M * ((a.N + 3) / 4);
     const int grid = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
     e = launch_pdl(split_reduce_kernel, dim3(grid), dim3(256), 0, s, nullptr, 0, static_cast<const float*>(w), ldw,
-                   splits, a.M, a.N, a.batch, a.alpha, a.beta, a.C, a.ldc, a.strideC, a.vecC, a);
+                   splits, a.M, a.N, a.batch, a.alpha, a.beta, a.C, a.ldc, a.strideC, a.vecC, chk);
   }
   cudaError_t ef = cudaFreeAsync(w, s);
   if (e == cudaSuccess) e = ef;
@@ -935,6 +945,9 @@ gemm_status_t kselect_conv3x3(gemm_handle_t h, const float* x, int32_t N, int32_
       cudaGetDevice(&dev) == cudaSuccess &&
       make_args('N', 'T', M, Cout, K, 1.f, x, K, weights, K, 0.f, out, Cout, 1, 4, &a, &noop) == GEMM_OK && !noop) {
     a.lda = C;  // of the image; its neighbourhoods are not stored
+#ifdef KS_DEBUG_BOUNDS
+    a.ext[0] = M * C * 4 - g_shrink[0];
+#endif
     const int sms = sm_count_of(dev);
     const double col_us = 2e6 * M * K * 4 / kSplitReduceBps;  // writing the neighbourhoods out and reading them back
     F32tcPlan plan;
