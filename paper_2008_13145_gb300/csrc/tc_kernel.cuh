@@ -424,7 +424,8 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, TF32>::THREADS, 1)
     int acc = 0;
     uint32_t acc_phase = 0;
     for (int tile = unit0; tile < p.num_tiles; tile += units) {
-      if (!mbar_wait(&accf_bar[acc], acc_phase, p.status, kStatusTimeoutAcc)) break;
+      const bool ok = mbar_wait(&accf_bar[acc], acc_phase, p.status, kStatusTimeoutAcc);
+      if (!__all_sync(0xffffffffu, ok)) break;  // a warp's lanes go on, or give up, together
       tc_fence_after();
       const TileLoc L = locate<GROUPED>(p, g, index, &tmA, &tmB, tile);
       const int quad = warp & 3, row0 = L.tm * kBM + quad * 32;
@@ -440,6 +441,7 @@ __global__ void __launch_bounds__(TcCfg<BN, STAGES, TF32>::THREADS, 1)
         tmem_ld_wait();
         if (row0 < L.M && L.tn * BN + c0 < L.N)
           store_chunk32<Cfg::STORE_COLS>(L, cbase, row0, L.tn * BN + c0, stage, r, lane);
+        __syncwarp();  // lanes past M return early; the next load and the fence want the whole warp
       }
       tc_fence_before();
       mbar_arrive(&acce_bar[acc]);
