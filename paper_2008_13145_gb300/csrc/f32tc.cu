@@ -324,6 +324,14 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int* s
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, code));
 }
 
+// The last chunks' slots are freed by commits that nobody else waits for; their
+// arrivals have to come (bounded) before the CTA that holds the barriers may exit.
+template <int STAGES>
+__device__ __forceinline__ void wait_freed(uint64_t* empty, int total, int* status) {
+  for (int i = max(0, total - STAGES); i < total; ++i)
+    if (!warp_wait(&empty[i % STAGES], (i / STAGES) & 1, status, kStatusTimeoutEmpty)) break;
+}
+
 struct Item {
   int b, m0, n0, kbeg, kend;
   int64_t slab;  // batch entry, or (batch entry, split) of the workspace
@@ -773,6 +781,7 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
       __syncwarp();
       if (lane == 0) mbar_arrive(&full[stage]);
     }
+    wait_freed<C::STAGES>(empty, total, p.status);
   } else {
     // ---------------------------------------------------------------- accumulators, C
     if constexpr (C::REGS_READ > kRegsLaunch) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::REGS_READ));
@@ -959,6 +968,7 @@ __device__ __forceinline__ void convert_pair(const Args& p, int total, bool is_a
     __syncwarp();
     if (lane == 0) arrive_cluster(in_cta(smem_u32(&full[stage]), 0));
   }
+  wait_freed<Pair::STAGES>(empty, total, p.status);
 }
 
 template <int AK, bool B_MN>
