@@ -694,11 +694,16 @@ gemm_status_t kselect_wait_selftest(int64_t limit_ns, int32_t* waited_out, void*
  * kselect_f32tc_choice returns the bn that a handle call uses instead of SIMT
  * config `config_id` (0: it runs the config), and the split factor, for these
  * sizes; `aligned` says whether every row allows 16-byte access.  Needs a GPU
- * for the occupancy query.  Negative gemm_status_t on error. */
+ * for the occupancy query.  Negative gemm_status_t on error.
+ * kselect_conv3x3_selftest runs kselect_conv3x3's product as the selftest does
+ * (C a multiple of 32, image and weights 16-byte aligned, else UNSUPPORTED). */
 gemm_status_t kselect_f32tc_selftest(int32_t bn, int32_t splits, char transA, char transB, int64_t M, int64_t N,
                                      int64_t K, float alpha, const float* A_dev, int64_t lda, int64_t strideA,
                                      const float* B_dev, int64_t ldb, int64_t strideB, float beta, float* C_dev,
                                      int64_t ldc, int64_t strideC, int64_t batch, void* stream);
+gemm_status_t kselect_conv3x3_selftest(int32_t bn, int32_t splits, const float* x_dev, int32_t N, int32_t H, int32_t W,
+                                       int32_t C, const float* weights_dev, int32_t Cout, const float* bias_dev,
+                                       int32_t relu, float* out_dev, void* stream);
 int32_t kselect_f32tc_choice(int32_t config_id, int64_t M, int64_t N, int64_t K, int64_t batch, int32_t transA,
                              int32_t aligned, int32_t* splits);
 

@@ -920,6 +920,31 @@ gemm_status_t gemm(gemm_handle_t h, char transA, char transB, int64_t M, int64_t
   return launch_selected(id, a, static_cast<cudaStream_t>(stream));
 }
 
+// The product of an image's neighbourhoods with the weights, the image itself as A;
+// false where the tensor-core kernel cannot read it.
+static bool conv_args(const float* x, int64_t M, int32_t C, const float* weights, int32_t Cout, float* out,
+                      GemmArgs* a) {
+  const int64_t K = 9LL * C;
+  bool noop = false;
+  if (C % 32 != 0 || (uintptr_t)x % 16 != 0 || (uintptr_t)weights % 16 != 0 ||
+      make_args('N', 'T', M, Cout, K, 1.f, x, K, weights, K, 0.f, out, Cout, 1, 4, a, &noop) != GEMM_OK || noop)
+    return false;
+  a->lda = C;  // of the image; its neighbourhoods are not stored
+#ifdef KS_DEBUG_BOUNDS
+  a->ext[0] = M * C * 4 - g_shrink[0];
+#endif
+  return true;
+}
+
+static gemm_status_t conv_run(const F32tcPlan& plan, const GemmArgs& a, int32_t H, int32_t W, int32_t C,
+                              const float* bias, int32_t relu, int sms, int* status, void* stream) {
+  const bool split = plan.splits > 1;  // the sum of the partials comes before bias and ReLU
+  const Conv3x3 conv{H, W, C, split ? nullptr : bias, split ? 0 : relu};
+  gemm_status_t st = f32tc_run(plan, a, sms, status, static_cast<cudaStream_t>(stream), &conv);
+  if (st != GEMM_OK || !split || (!bias && !relu)) return st;
+  return kselect_bias_act(a.C, a.M, a.N, a.ldc, bias, relu, stream);
+}
+
 gemm_status_t kselect_conv3x3(gemm_handle_t h, const float* x, int32_t N, int32_t H, int32_t W, int32_t C,
                               const float* weights, int32_t Cout, const float* bias, int32_t relu, float* col,
                               int64_t ld, float* out, void* stream) {
@@ -939,31 +964,23 @@ gemm_status_t kselect_conv3x3(gemm_handle_t h, const float* x, int32_t N, int32_
     return GEMM_OK;
   }
   GemmArgs a;
-  bool noop = false;
   int dev = 0;
-  if (fp32 && C % 32 == 0 && (uintptr_t)x % 16 == 0 && (uintptr_t)weights % 16 == 0 &&
-      cudaGetDevice(&dev) == cudaSuccess &&
-      make_args('N', 'T', M, Cout, K, 1.f, x, K, weights, K, 0.f, out, Cout, 1, 4, &a, &noop) == GEMM_OK && !noop) {
-    a.lda = C;  // of the image; its neighbourhoods are not stored
-#ifdef KS_DEBUG_BOUNDS
-    a.ext[0] = M * C * 4 - g_shrink[0];
-#endif
+  if (fp32 && conv_args(x, M, C, weights, Cout, out, &a) && cudaGetDevice(&dev) == cudaSuccess) {
     const int sms = sm_count_of(dev);
     const double col_us = 2e6 * M * K * 4 / kSplitReduceBps;  // writing the neighbourhoods out and reading them back
     F32tcPlan plan;
     int* status = f32tc_plan(id, a, dev, sms, col_us, &plan) ? status_word_for(s) : nullptr;
-    if (status) {
-      const bool split = plan.splits > 1;  // the sum of the partials comes before bias and ReLU
-      const Conv3x3 conv{H, W, C, split ? nullptr : bias, split ? 0 : relu};
-      gemm_status_t st = f32tc_run(plan, a, sms, status, s, &conv);
-      if (st != GEMM_OK || !split || (!bias && !relu)) return st;
-      return kselect_bias_act(out, M, Cout, Cout, bias, relu, stream);
-    }
+    if (status) return conv_run(plan, a, H, W, C, bias, relu, sms, status, stream);
   }
   gemm_status_t st = kselect_im2col3x3(x, N, H, W, C, col, ld, stream);
   if (st == GEMM_OK) st = gemm(h, 'N', 'T', M, Cout, K, 1.f, col, ld, weights, K, 0.f, out, Cout, 1, stream);
   if (st == GEMM_OK && (bias || relu)) st = kselect_bias_act(out, M, Cout, Cout, bias, relu, stream);
   return st;
+}
+
+static F32tcPlan forced_plan(int bn, int splits, int64_t K) {
+  const int64_t kc = ceil_div(ceil_div(K, splits), kF32tcChunk) * kF32tcChunk;
+  return F32tcPlan{bn, (int)ceil_div(K, kc), (int)kc};
 }
 
 gemm_status_t kselect_f32tc_selftest(int32_t bn, int32_t splits, char transA, char transB, int64_t M, int64_t N,
@@ -981,9 +998,21 @@ gemm_status_t kselect_f32tc_selftest(int32_t bn, int32_t splits, char transA, ch
   cudaError_t e = cudaGetDevice(&dev);
   int* status = e == cudaSuccess ? tc_status_word() : nullptr;
   if (!status) { set_last_cuda_error(e != cudaSuccess ? e : cudaGetLastError()); return GEMM_ERR_CUDA; }
-  const int64_t kc = ceil_div(ceil_div(K, splits), kF32tcChunk) * kF32tcChunk;
-  const F32tcPlan plan{bn, (int)ceil_div(K, kc), (int)kc};
-  return f32tc_run(plan, a, sm_count_of(dev), status, static_cast<cudaStream_t>(stream));
+  return f32tc_run(forced_plan(bn, splits, K), a, sm_count_of(dev), status, static_cast<cudaStream_t>(stream));
+}
+
+gemm_status_t kselect_conv3x3_selftest(int32_t bn, int32_t splits, const float* x, int32_t N, int32_t H, int32_t W,
+                                       int32_t C, const float* weights, int32_t Cout, const float* bias, int32_t relu,
+                                       float* out, void* stream) {
+  if ((bn != 64 && bn != 128 && bn != 256) || splits < 1 || splits > kSplitMaxFactor) return GEMM_ERR_INVALID_ARG;
+  if (N < 1 || H < 1 || W < 1 || C < 1 || Cout < 1 || !x || !weights || !out) return GEMM_ERR_INVALID_ARG;
+  GemmArgs a;
+  if (!conv_args(x, (int64_t)N * H * W, C, weights, Cout, out, &a) || a.K > kF32tcMaxK) return GEMM_ERR_UNSUPPORTED;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  int* status = e == cudaSuccess ? tc_status_word() : nullptr;
+  if (!status) { set_last_cuda_error(e != cudaSuccess ? e : cudaGetLastError()); return GEMM_ERR_CUDA; }
+  return conv_run(forced_plan(bn, splits, a.K), a, H, W, C, bias, relu, sm_count_of(dev), status, stream);
 }
 
 int32_t kselect_f32tc_choice(int32_t id, int64_t M, int64_t N, int64_t K, int64_t batch, int32_t transA,

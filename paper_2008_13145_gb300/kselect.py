@@ -99,6 +99,7 @@ _sig("gemm_grouped_reserve", i32, [vp, i32, ctypes.POINTER(Problem), i32])
 _sig("gemm_grouped_select", i32, [vp, i32, ctypes.POINTER(Problem)])
 _sig("kselect_f32tc_selftest", i32, [i32, i32, ch, ch, i64, i64, i64, f32, vp, i64, i64, vp, i64, i64, f32, vp, i64,
                                      i64, i64, vp])
+_sig("kselect_conv3x3_selftest", i32, [i32, i32, vp, i32, i32, i32, i32, vp, i32, vp, i32, vp, vp])
 _sig("kselect_f32tc_choice", i32, [i32, i64, i64, i64, i64, i32, i32, ctypes.POINTER(i32)])
 _sig("mlp_features", i32, [i32, vp, vp, vp])
 _sig("mlp_forward", i32, [i32, vp, vp, vp, vp])
@@ -394,6 +395,12 @@ def f32tc_selftest(bn: int, splits: int, transA: str, transB: str, M, N, K, alph
     check(_lib.kselect_f32tc_selftest(bn, splits, _c(transA), _c(transB), M, N, K, alpha, ptr(A), lda, strideA, ptr(B),
                                       ldb, strideB, beta, ptr(C), ldc, strideC, batch, stream_handle(stream)),
           "kselect_f32tc_selftest")
+
+
+def conv3x3_selftest(bn: int, splits: int, x, N, H, W, C, weights, Cout, bias, relu, out, stream=None) -> None:
+    """conv3x3 on the tensor cores with bn-wide tiles and up to `splits` K ranges, whatever conv3x3() would choose."""
+    check(_lib.kselect_conv3x3_selftest(bn, splits, ptr(x), N, H, W, C, ptr(weights), Cout, ptr(bias), int(relu),
+                                        ptr(out), stream_handle(stream)), "kselect_conv3x3_selftest")
 
 
 def f32tc_choice(cid: int, M, N, K, batch=1, transA="N", aligned=True) -> tuple[int, int]:
@@ -766,7 +773,7 @@ def exported_symbols() -> list[str]:
             "kselect_debug_shrink_extents", "gemm_config_count", "gemm_config_id",
             "gemm_config_params", "gemm_split_choose", "gemm_split_factor", "gemm_library_create", "gemm_library_destroy", "select_kernel", "gemm",
             "gemm_with_config", "gemm_host_pipeline", "gemm_strided_batched", "gemm_strided_batched_with_config", "gemm_host", "gemm_benchmark", "gemm_error_check", "kselect_fill_uniform",
-            "gemm_benchmark_configs", "gemm_device_status", "kselect_wait_selftest", "kselect_f32tc_selftest", "kselect_f32tc_choice", "kselect_normalise", "kselect_kmeans", "kselect_score",
+            "gemm_benchmark_configs", "gemm_device_status", "kselect_wait_selftest", "kselect_f32tc_selftest", "kselect_conv3x3_selftest", "kselect_f32tc_choice", "kselect_normalise", "kselect_kmeans", "kselect_score",
             "kselect_im2col3x3", "kselect_conv3x3", "kselect_bias_act", "kselect_maxpool2x2", "kselect_im2col3x3_nchw", "kselect_bias_act_nchw", "kselect_knn", "kselect_representatives", "kselect_top_n", "kselect_tree_regress", "kselect_tree_train", "kselect_tree_train_rf", "kselect_spectral_embedding", "kselect_cluster_geomean", "kselect_pca", "kselect_pca_backproject", "mlp_features", "mlp_forward", "mlp_loss_grad",
             "mlp_adam_step", "mlp_loss_grad_noalloc", "mlp_train", "select_kernels_batched", "gemm_grouped_plan_create", "gemm_grouped_run",
             "gemm_grouped_plan_destroy", "gemm_grouped", "gemm_grouped_with_config", "gemm_grouped_reserve",
