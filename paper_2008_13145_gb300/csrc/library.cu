@@ -419,7 +419,8 @@ static double f32tc_cost(const F32tcCost& c, const GemmArgs& a, int64_t tiles, i
 // chain rounds once per K; the tensor cores' chunk sums carry a truncation of
 // 0.86 2^-24 on average, and a rounding per chunk.  A plan is considered only
 // where it is the more exact one; on signed data it then is by a factor of 1.4
-// to 7 (all of the 500 shapes).
+// to 7 (all of the 500 shapes).  The rule is about dense rows: the host does not
+// know the values (see f32tc.cu for rows with few non-zero terms).
 static double f32tc_error(double K, int S) { return 1.13 + 0.0015 * K / ((double)S * S) + (S > 1 ? 0.04 * S : 0.0); }
 static double simt_error(double K, int S) { return 0.05 * K / ((double)S * S) + (S > 1 ? 0.07 * S : 0.0); }
 
