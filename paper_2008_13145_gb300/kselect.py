@@ -647,15 +647,15 @@ assert _pack_problem.size == ctypes.sizeof(Problem)
 def _problems(problems):
     """problems: iterable of dicts with M, N, K, transA, transB, alpha, beta, A, lda, B, ldb, C, ldc."""
     arr = (Problem * len(problems))()
-    pack, at = _pack_problem.pack_into, 0
-    try:
-        for q in problems:
-            pack(arr, at, q["M"], q["N"], q["K"], _c(q.get("transA", "N")), _c(q.get("transB", "T")),
-                 q.get("alpha", 1.0), q.get("beta", 0.0), ptr(q["A"]) or 0, q["lda"], ptr(q["B"]) or 0, q["ldb"],
-                 ptr(q["C"]) or 0, q["ldc"])
-            at += _pack_problem.size
-    except struct.error as e:
-        raise TypeError(str(e)) from e
+    pack, size = _pack_problem.pack_into, _pack_problem.size
+    for i, q in enumerate(problems):
+        a, b, c, ta, tb = ptr(q["A"]), ptr(q["B"]), ptr(q["C"]), _c(q.get("transA", "N")), _c(q.get("transB", "T"))
+        alpha, beta = q.get("alpha", 1.0), q.get("beta", 0.0)
+        try:
+            pack(arr, i * size, q["M"], q["N"], q["K"], ta, tb, alpha, beta, a or 0, q["lda"], b or 0, q["ldb"], c or 0,
+                 q["ldc"])
+        except (struct.error, OverflowError):  # what pack refuses, ctypes may take (alpha past FP32's range) or name
+            arr[i] = Problem(q["M"], q["N"], q["K"], ta, tb, alpha, beta, a, q["lda"], b, q["ldb"], c, q["ldc"])
     return arr
 
 
