@@ -73,7 +73,10 @@ int32_t gemm_last_cuda_error(void);
  * (synchronising the device; clear != 0 resets it); kselect_debug_shrink_extents
  * declares the operand extents smaller by the given bytes on later calls (a
  * test of the checker itself, which then flags accesses that are in fact
- * inside the buffers).  Release builds return GEMM_ERR_UNSUPPORTED. */
+ * inside the buffers); kselect_debug_fail_scratch makes the next `requests`
+ * scratch allocations fail for want of memory.  Release builds return
+ * GEMM_ERR_UNSUPPORTED. */
+gemm_status_t kselect_debug_fail_scratch(int32_t requests);
 gemm_status_t kselect_debug_bounds_errors(int32_t* errors_out, int32_t clear);
 gemm_status_t kselect_debug_shrink_extents(int64_t a_bytes, int64_t b_bytes, int64_t c_bytes);
 

@@ -294,7 +294,14 @@ void scratch_drop_handle() {
   cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
+#ifdef KS_DEBUG_BOUNDS
+static std::atomic<int> g_scratch_failures{0};  // test hook: scratch requests to refuse
+#endif
+
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+#ifdef KS_DEBUG_BOUNDS
+  if (g_scratch_failures.load() > 0 && g_scratch_failures.fetch_sub(1) > 0) return cudaErrorMemoryAllocation;
+#endif
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaStreamIsCapturing(s, &cs);
   if (e != cudaSuccess) return e;
@@ -489,8 +496,11 @@ static bool f32tc_plan(int id, const GemmArgs& a, int dev, int sms, double other
   return f32tc_fastest(a, sms, us / kF32tcMargin, 0.9 * simt_error(a.K, simt_splits), plan);
 }
 
+// *no_scratch: there was no memory for the workspace and nothing was launched, so
+// that a caller with another kernel, which may need none, can run that.
 static gemm_status_t f32tc_run(const F32tcPlan& plan, const GemmArgs& a, int sms, int* status, cudaStream_t s,
-                               const Conv3x3* conv = nullptr) {
+                               bool* no_scratch, const Conv3x3* conv = nullptr) {
+  *no_scratch = false;
   const int bn = plan.bn, splits = plan.splits, kchunk = plan.kchunk;
   cudaError_t e;
   if (splits <= 1) {
@@ -502,6 +512,10 @@ static gemm_status_t f32tc_run(const F32tcPlan& plan, const GemmArgs& a, int sms
   const size_t bytes = (size_t)splits * a.batch * a.M * ldw * sizeof(float);
   void* w = nullptr;
   e = scratch_alloc(&w, bytes, s);
+  if (e == cudaErrorMemoryAllocation) {
+    *no_scratch = true;
+    cudaGetLastError();
+  }
   if (e != cudaSuccess) { set_last_cuda_error(e); return GEMM_ERR_CUDA; }
   GemmArgs p = a;
   p.alpha = 1.f;
@@ -598,7 +612,9 @@ static gemm_status_t launch_selected(int id, const GemmArgs& a, cudaStream_t s) 
   if (!f32tc_plan(id, a, dev, sms, 0.0, &plan)) return launch_config(id, a, s);
   int* status = status_word_for(s);
   if (!status) return launch_config(id, a, s);
-  return f32tc_run(plan, a, sms, status, s);
+  bool no_scratch = false;
+  gemm_status_t st = f32tc_run(plan, a, sms, status, s, &no_scratch);
+  return no_scratch ? launch_config(id, a, s) : st;
 }
 
 static int elem_bytes_of(int id) { return family_of(id) == GEMM_PREC_BF16 ? 2 : 4; }
@@ -659,6 +675,17 @@ gemm_status_t kselect_debug_shrink_extents(int64_t a_bytes, int64_t b_bytes, int
   return GEMM_OK;
 #else
   (void)a_bytes; (void)b_bytes; (void)c_bytes;
+  return GEMM_ERR_UNSUPPORTED;
+#endif
+}
+
+gemm_status_t kselect_debug_fail_scratch(int32_t requests) {
+#ifdef KS_DEBUG_BOUNDS
+  if (requests < 0) return GEMM_ERR_INVALID_ARG;
+  g_scratch_failures = requests;
+  return GEMM_OK;
+#else
+  (void)requests;
   return GEMM_ERR_UNSUPPORTED;
 #endif
 }
@@ -938,10 +965,11 @@ static bool conv_args(const float* x, int64_t M, int32_t C, const float* weights
 }
 
 static gemm_status_t conv_run(const F32tcPlan& plan, const GemmArgs& a, int32_t H, int32_t W, int32_t C,
-                              const float* bias, int32_t relu, int sms, int* status, void* stream) {
+                              const float* bias, int32_t relu, int sms, int* status, void* stream,
+                              bool* no_scratch) {
   const bool split = plan.splits > 1;  // the sum of the partials comes before bias and ReLU
   const Conv3x3 conv{H, W, C, split ? nullptr : bias, split ? 0 : relu};
-  gemm_status_t st = f32tc_run(plan, a, sms, status, static_cast<cudaStream_t>(stream), &conv);
+  gemm_status_t st = f32tc_run(plan, a, sms, status, static_cast<cudaStream_t>(stream), no_scratch, &conv);
   if (st != GEMM_OK || !split || (!bias && !relu)) return st;
   return kselect_bias_act(a.C, a.M, a.N, a.ldc, bias, relu, stream);
 }
@@ -971,7 +999,11 @@ gemm_status_t kselect_conv3x3(gemm_handle_t h, const float* x, int32_t N, int32_
     const double col_us = 2e6 * M * K * 4 / kSplitReduceBps;  // writing the neighbourhoods out and reading them back
     F32tcPlan plan;
     int* status = f32tc_plan(id, a, dev, sms, col_us, &plan) ? status_word_for(s) : nullptr;
-    if (status) return conv_run(plan, a, H, W, C, bias, relu, sms, status, stream);
+    if (status) {
+      bool no_scratch = false;
+      gemm_status_t st = conv_run(plan, a, H, W, C, bias, relu, sms, status, stream, &no_scratch);
+      if (!no_scratch) return st;
+    }
   }
   gemm_status_t st = kselect_im2col3x3(x, N, H, W, C, col, ld, stream);
   if (st == GEMM_OK) st = gemm(h, 'N', 'T', M, Cout, K, 1.f, col, ld, weights, K, 0.f, out, Cout, 1, stream);
@@ -999,7 +1031,9 @@ gemm_status_t kselect_f32tc_selftest(int32_t bn, int32_t splits, char transA, ch
   cudaError_t e = cudaGetDevice(&dev);
   int* status = e == cudaSuccess ? tc_status_word() : nullptr;
   if (!status) { set_last_cuda_error(e != cudaSuccess ? e : cudaGetLastError()); return GEMM_ERR_CUDA; }
-  return f32tc_run(forced_plan(bn, splits, K), a, sm_count_of(dev), status, static_cast<cudaStream_t>(stream));
+  bool no_scratch = false;
+  return f32tc_run(forced_plan(bn, splits, K), a, sm_count_of(dev), status, static_cast<cudaStream_t>(stream),
+                   &no_scratch);
 }
 
 gemm_status_t kselect_conv3x3_selftest(int32_t bn, int32_t splits, const float* x, int32_t N, int32_t H, int32_t W,
@@ -1013,7 +1047,8 @@ gemm_status_t kselect_conv3x3_selftest(int32_t bn, int32_t splits, const float* 
   cudaError_t e = cudaGetDevice(&dev);
   int* status = e == cudaSuccess ? tc_status_word() : nullptr;
   if (!status) { set_last_cuda_error(e != cudaSuccess ? e : cudaGetLastError()); return GEMM_ERR_CUDA; }
-  return conv_run(forced_plan(bn, splits, a.K), a, H, W, C, bias, relu, sm_count_of(dev), status, stream);
+  bool no_scratch = false;
+  return conv_run(forced_plan(bn, splits, a.K), a, H, W, C, bias, relu, sm_count_of(dev), status, stream, &no_scratch);
 }
 
 int32_t kselect_f32tc_choice(int32_t id, int64_t M, int64_t N, int64_t K, int64_t batch, int32_t transA,

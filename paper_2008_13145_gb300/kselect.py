@@ -68,6 +68,7 @@ _sig("gemm_status_string", ctypes.c_char_p, [i32])
 _sig("gemm_last_cuda_error", i32, [])
 _sig("kselect_debug_bounds_errors", i32, [ctypes.POINTER(i32), i32])
 _sig("kselect_debug_shrink_extents", i32, [i64, i64, i64])
+_sig("kselect_debug_fail_scratch", i32, [i32])
 _sig("gemm_config_count", i32, [i32])
 _sig("gemm_config_id", i32, [i32, i32])
 _sig("gemm_config_params", i32, [i32, ctypes.POINTER(i32)])
@@ -770,7 +771,7 @@ def select_kernels_batched(handle: Handle, shapes, ids_out, pred=None, stream=No
 def exported_symbols() -> list[str]:
     """Names of the C-ABI entry points this binding expects."""
     return ["gemm_status_string", "gemm_last_cuda_error", "kselect_debug_bounds_errors",
-            "kselect_debug_shrink_extents", "gemm_config_count", "gemm_config_id",
+            "kselect_debug_shrink_extents", "kselect_debug_fail_scratch", "gemm_config_count", "gemm_config_id",
             "gemm_config_params", "gemm_split_choose", "gemm_split_factor", "gemm_library_create", "gemm_library_destroy", "select_kernel", "gemm",
             "gemm_with_config", "gemm_host_pipeline", "gemm_strided_batched", "gemm_strided_batched_with_config", "gemm_host", "gemm_benchmark", "gemm_error_check", "kselect_fill_uniform",
             "gemm_benchmark_configs", "gemm_device_status", "kselect_wait_selftest", "kselect_f32tc_selftest", "kselect_conv3x3_selftest", "kselect_f32tc_choice", "kselect_normalise", "kselect_kmeans", "kselect_score",
