@@ -274,10 +274,12 @@ def run_ours(args, ws, rank, local):
     # first loads the kernels the deployment does not use, the next ones are timed).
     per_launch_ms(best_cfg)
     exh_ms = per_launch_median(best_cfg)
-    ratio = np.minimum(exh_ms / sel_ms, 1.0)
+    # Both sides as configs: the sweep knows nothing of the tensor cores that gemm() may use instead.
+    per_launch_ms(chosen)
+    ratio = np.minimum(exh_ms / per_launch_median(chosen), 1.0)
     live = {"geomean": float(np.exp(np.mean(np.log(ratio)))), "mean": float(np.mean(ratio)),
             "source": "per-shape launch times this run, median of 3 passes each: exhaustive-best config vs "
-                      "selected config"}
+                      "selected config, each run as named (gemm() runs some on the tensor cores at FP32 accuracy)"}
     # Dominant kernel: the one with the largest share of step time.
     by_cfg = {}
     for c, t, sh in zip(ran, sel_ms, shapes):
@@ -464,7 +466,9 @@ def tc_families(args, ks, tune, shapes, te, bufs, stream, dev):
 
         for _ in range(args.warmup):
             run()
-        sel = np.median([per_launch() for _ in range(3)], axis=0)
+        picked = [ks.select_kernel(h, sh.M, sh.N, sh.K, sh.batch) for sh in shapes]
+        run(picked)  # loads configs that gemm() leaves to the tensor cores
+        sel = np.median([per_launch(picked) for _ in range(3)], axis=0)
         run(best)  # loads the kernels the deployment does not use
         exh = np.median([per_launch(best) for _ in range(3)], axis=0)
         ratio = np.minimum(exh / sel, 1.0)
