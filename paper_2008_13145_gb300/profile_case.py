@@ -1,9 +1,11 @@
 """Run one kernel configuration on one GEMM size a few times (an ncu target).
 
     python -m paper_2008_13145_gb300.profile_case --config 531 --shape 4096 4096 4096 1 N N --reps 3
+    python -m paper_2008_13145_gb300.profile_case --f32tc 256 1 --shape 4096 4096 4096 1 N N --reps 3
     python -m paper_2008_13145_gb300.profile_case --grouped 1216 --reps 2
     python -m paper_2008_13145_gb300.profile_case --vendor-fp32 --shape 4096 4096 4096 1 N N --reps 2
 
+--f32tc runs the FP32 product on the tensor cores with that tile width and K split.
 --vendor-fp32 runs the vendor library's FP32 GEMM instead (torch.mm with TF32
 off, a batch-1 NN product only): a reference point for profiling, not part of
 the library.
@@ -26,6 +28,7 @@ def main(argv=None):
     ap.add_argument("--config", type=int)
     ap.add_argument("--shape", nargs=6, metavar=("M", "N", "K", "BATCH", "TA", "TB"))
     ap.add_argument("--grouped", type=int, help="config id: run the 256-problem grouped workload")
+    ap.add_argument("--f32tc", type=int, nargs=2, metavar=("BN", "SPLITS"))
     ap.add_argument("--vendor-fp32", action="store_true", help="time torch.mm (cuBLAS FP32, TF32 off) instead")
     ap.add_argument("--reps", type=int, default=3)
     a = ap.parse_args(argv)
@@ -62,11 +65,16 @@ def main(argv=None):
     else:
         M, N, K, b = (int(x) for x in a.shape[:4])
         sh = wl.Shape(M, N, K, b, a.shape[4], a.shape[5])
-        A, B, C, lda, ldb, ldc = tune.alloc_inputs(sh, ks.family_of(a.config), 1)
+        A, B, C, lda, ldb, ldc = tune.alloc_inputs(sh, ks.PREC_F32 if a.f32tc else ks.family_of(a.config), 1)
         flops = sh.flops
         for _ in range(a.reps):
             e0.record()
-            ks.gemm_with_config(a.config, sh.transA, sh.transB, M, N, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, b)
+            if a.f32tc:
+                ks.f32tc_selftest(*a.f32tc, sh.transA, sh.transB, M, N, K, 1.0, A, lda,
+                                  lda * (M if sh.transA == "N" else K), B, ldb, ldb * (K if sh.transB == "N" else N), 0.0,
+                                  C, ldc, ldc * M, b)
+            else:
+                ks.gemm_with_config(a.config, sh.transA, sh.transB, M, N, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, b)
             e1.record()
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1)
