@@ -330,10 +330,13 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int* s
 
 // The last chunks' slots are freed by commits that nobody else waits for; their
 // arrivals have to come (bounded) before the CTA that holds the barriers may exit.
+// The issuing thread waits for its own (in the converting warps the wait cost
+// registers that spill: 323 x 312 x 3945 x 8 A^T B 89 us instead of 83), the pair's
+// converting warps for the first CTA's.
 template <int STAGES>
 __device__ __forceinline__ void wait_freed(uint64_t* empty, int total, int* status) {
   for (int i = max(0, total - STAGES); i < total; ++i)
-    if (!warp_wait(&empty[i % STAGES], (i / STAGES) & 1, status, kStatusTimeoutEmpty)) break;
+    if (!mbar_wait(&empty[i % STAGES], (i / STAGES) & 1, status, kStatusTimeoutEmpty)) break;
 }
 
 struct Item {
@@ -710,6 +713,7 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
         if (!mbar_wait(&full[stage], (i / C::STAGES) & 1, p.status, kStatusTimeoutFull)) break;
         issue_mmas<BN>(smem + stage * C::STAGE, tmem + (uint32_t)((i & 1) * BN), &empty[stage], &accf[i & 1]);
       }
+      wait_freed<C::STAGES>(empty, total, p.status);
     }
   } else if (warp >= kReaders) {
     // ---------------------------------------------------------------- load and convert
@@ -785,7 +789,6 @@ __global__ void __launch_bounds__(kThreads, 1) f32tc_kernel(const __grid_constan
       __syncwarp();
       if (lane == 0) mbar_arrive(&full[stage]);
     }
-    wait_freed<C::STAGES>(empty, total, p.status);
   } else {
     // ---------------------------------------------------------------- accumulators, C
     if constexpr (C::REGS_READ > kRegsLaunch) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::REGS_READ));
