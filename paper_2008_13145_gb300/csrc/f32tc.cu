@@ -16,9 +16,10 @@
 // against 0.41.  Products by 0, by powers of two and of integers are exact.
 //
 // Bound: six 16-bit products, 315 TFLOP/s of the measured BF16 rate; the FP32
-// pipe's peak is 80.  4096 x 4096 x 4096: 625 us, 220 TFLOP/s (A B^T 590 us, 233;
-// the last of four rounds of 256 x 256 tiles is a third full: 277 at 4864 x 4096 x
-// 4096) against 2,520 us for the SIMT kernel.  What holds it is the converting
+// pipe's peak is 80.  4096 x 4096 x 4096: 572 us, 240 TFLOP/s (A B^T 547; up to 10 %
+// more once the clocks fall under the power cap; the last of four rounds of 256 x
+// 256 tiles is a third full: 4864 x 4096 x 4096 takes as long, 285 TFLOP/s) against
+// 2,525 us for the SIMT kernel.  What holds it is the converting
 // warps' chain of latencies (load, split, store, fence per chunk), then
 // shared-memory bandwidth: the MMAs of 128-wide tiles alone read 128 bytes a clock.
 //
@@ -29,9 +30,9 @@
 // its part of such a tile unwritten and marks it; when all of the CTA's chunks
 // are summed, so that no role waits, the reading warps compute the marked parts
 // by plain FP32 FMAs over K (redo), so such inputs give what the FP32 SIMT family
-// gives.  One NaN takes 2048 x 2048 x 2048 from 85 to 563 us (SIMT kernel: 366, on
-// any values), an infinity in every row of 4096 x 4096 x 4096 from 595 to 4,410
-// (SIMT: 2,530): the parts of a tile stay with its SM.  (Computed where they were
+// gives.  One NaN takes 2048 x 2048 x 2048 from 83 to 564 us (SIMT kernel: 365, on
+// any values), an infinity in every row of 4096 x 4096 x 4096 from 578 to 4,400
+// (SIMT: 2,525): the parts of a tile stay with its SM.  (Computed where they were
 // met, by lanes with a row each: 11,640 and 101,000 us.)
 //
 // One persistent CTA per SM, five warpgroups.
@@ -75,7 +76,7 @@ constexpr int kMaxItems = 1024;               // items of one CTA or pair: a byt
 
 // Stages: what fits in 164 KB, so that 92 KB are left as L1, where the FP32
 // loads under way land (with 28 KB left, the 256 x 256 tiles of 4096 x 4096 x
-// 4096 took 838 us against 659).
+// 4096 took 27 % longer).
 template <int BN>
 struct Cfg {
   static constexpr int A_PART = kBM * 64;  // bytes of one part of a slice
@@ -86,8 +87,8 @@ struct Cfg {
   static constexpr int TMEM = 2 * BN;  // two accumulators
   static constexpr int G = BN / 8;     // accumulator columns per reading warp and quarter
   // 128 x 32 + 256 x (112 + 112) or 256 x (128 + 96): at BN 128 a reading thread
-  // holds 64 accumulators (with 96 registers it spills: 896 us against 674 at
-  // 4096 x 4096 x 4096, A B^T), at BN 64 the converting ones gain more.
+  // holds 64 accumulators (with 96 registers it spills: a third slower at 4096 x
+  // 4096 x 4096, A B^T), at BN 64 the converting ones gain more.
   static constexpr int REGS_CONVERT = BN == 128 ? 112 : 128, REGS_READ = BN == 128 ? 112 : 96;
 };
 
@@ -580,8 +581,8 @@ __device__ __forceinline__ void redo_block(const Args& p, const Item& it, int ro
                    INNER || (col + 4 * e + four < g.N && kk < left));
     }
   };
-  // (Not with A^T: the pair kernel of A^T B then takes 720 us at 4096 x 4096 x 4096
-  // on values that all split, 581 without.)
+  // (Not with A^T: the pair kernel of A^T B then takes 24 % longer at 4096 x 4096 x
+  // 4096 on values that all split.)
   const bool whole = AK != kCols && row0 + 4 * 31 < g.M && col + CW <= g.N;
   auto load = [&](int step) {
     const int k0 = it.kbeg + step * R::K;
@@ -945,9 +946,9 @@ __device__ __forceinline__ void convert_pair(const Args& p, int total, bool is_a
     uint32_t rem = 0;
     const uint32_t at = smem + stage * Pair::STAGE + (is_a ? 0 : kParts * Pair::PART);
     // Registers are reloaded as soon as they are stored: after each half of the
-    // eight K-contiguous parts (4096 x 4096 x 4096, A B^T: 578 us, 638 with the
-    // loads after all parts, 728 after each), after both MN-contiguous ones
-    // (A B: 641 us, 697 after each).
+    // eight K-contiguous parts (4096 x 4096 x 4096, A B^T: 10 % slower with the
+    // loads after all parts, 26 % after each), after both MN-contiguous ones
+    // (A B: 9 % slower after each).
     constexpr int H = S::PARTS == 8 ? 4 : S::PARTS;
     if (more && inner && left >= kBK) {
 #pragma unroll
