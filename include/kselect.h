@@ -206,8 +206,8 @@ int32_t select_kernel(gemm_handle_t handle, int64_t M, int64_t N, int64_t K, int
  * with a handle run that, at sizes where it is the more exact of the two on
  * dense operands.  Rows with fewer than about 24 non-zero terms are more exact
  * as FMA chains (one term: up to 2.6 units of 2^-24 |xy| against 1), and values
- * that do not split (NaN, infinities, magnitudes below about 2^-110) take 1.3 to
- * 2 times the SIMT kernel's time; gemm_with_config and its kin run the config
+ * that do not split (NaN, infinities, magnitudes below about 2^-110) take up to
+ * twice the SIMT kernel's time; gemm_with_config and its kin run the config
  * named.  A and B are float* for F32/TF32/F32X3 handles and bf16 (uint16_t*)
  * for BF16 handles.  M, N or batch == 0 is a no-op; K == 0
  * sets C = beta * C.  When beta == 0, C is only written (it may hold NaN).
